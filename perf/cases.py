@@ -222,10 +222,12 @@ def _batch_requests(case):
 
 
 def _toggles(case):
-    """The member ids that each session toggles on every request."""
+    """The member ids that each session toggles on every request, and those it holds at the start (half of all)."""
     rng = random.Random(case["mix"])
     total = case["resident"] + case["overflow"]
-    return [sorted(rng.sample(range(total), min(total, _log_int(rng, 8, case["toggle_max"])))) for _ in range(case["sessions"])]
+    toggles = [sorted(rng.sample(range(total), min(total, _log_int(rng, 8, case["toggle_max"])))) for _ in range(case["sessions"])]
+    held = [sorted(rng.sample(range(total), total // 2)) for _ in range(case["sessions"])]
+    return toggles, held
 
 
 def _composite(case):
@@ -299,7 +301,10 @@ def _prepare_serve(case, gen):
     server = binding.Server(resident[:, :, :row], overflow[:, :, :row], mask_format=case["data"], width=w if bits else None)
     sessions = [server.open_session() for _ in range(case["sessions"])]
     flat, views = _image_set([(w, h)] * len(sessions), counts=True, histogram=True)
-    toggles = [np.asarray(t, dtype=np.int32) for t in _toggles(case)]
+    toggles, held = ([np.asarray(t, dtype=np.int32) for t in sets] for sets in _toggles(case))
+    for session, ids in zip(sessions, held):
+        server.request(session, ids)
+    server.drain()
     return {"kind": "serve", "server": server, "sessions": sessions, "toggles": toggles, "views": views, "out": flat}
 
 
@@ -356,7 +361,7 @@ def work(case):
     px = case["width"] * case["height"]
     if kind == "serve":
         row = _row_bytes(case["data"], case["width"]) * case["height"]
-        toggles = _toggles(case)
+        toggles, _ = _toggles(case)
         outputs = 9 * px + 2048
         planes = 8 * px   # each session's composite, updated in place
         return {"bytes": sum(len(t) for t in toggles) * row + len(toggles) * (outputs + planes), "flops": 0}
