@@ -54,7 +54,7 @@ enum {
 typedef struct composite_engine_config {
     void *cuda_stream;        /* cudaStream_t for all engine work, NULL = the legacy
                                  default stream (ordered with the caller's work there) */
-    int32_t slab_members;     /* members per work item, 1..255; 0 = 128               */
+    int32_t slab_members;     /* most members of an op per work item, 1..255; 0 = 128  */
     int32_t ctas_per_sm;      /* persistent CTAs of 256 threads per SM, 1..8; 0 = 5   */
     int64_t wait_timeout_ms;  /* bound on host waits; 0 = 10000                        */
     int32_t schedule;         /* CPT_SCHEDULE_*; default CPT_SCHEDULE_PERSISTENT       */
@@ -63,10 +63,12 @@ typedef struct composite_engine_config {
                                  that streams its own rasters on a copy stream passes
                                  it here so the small uploads queue behind its uploads
                                  in order instead of competing for a copy engine      */
-    int32_t item_member_groups; /* work item size: a lane folds about this many
+    int32_t item_member_groups; /* work item size: a lane folds at most about this many
                                  (member, 16-pixel group) pairs per item, so an item
-                                 covers 32 x (item_member_groups / slab) groups of one
-                                 slab; 16..8192, 0 = 512                                */
+                                 covers up to 32 x (item_member_groups / slab) groups
+                                 of one slab (fewer when a submit would otherwise give
+                                 the launch's warps fewer than four items each);
+                                 16..8192, 0 = 512                                      */
     int32_t staging_buffers;  /* staging buffers for host ops, 2..8; 0 = 2           */
     int64_t staging_bytes;    /* bytes per staging buffer, >= 1 MiB (and >= the largest
                                  host raster); 0 = 256 MiB.  Allocated at the first
@@ -138,7 +140,11 @@ int composite_engine_clear_many(composite_engine *eng, const int32_t *planes, in
  * sign not +-1, N of a plane would go negative or above its count type's
  * maximum (2^32-1, or 65535 for a 16-bit plane), bad strides).
  * A pixel count that would go below zero raises the plane's underflow state
- * (reported by composite_engine_sync).
+ * (reported by composite_engine_sync).  A plane's device ops fold in list
+ * order while each holds at most slab_members members and they hold at most
+ * max(slab_members, item_member_groups) together, all in one mask format;
+ * beyond that they fold at the same time, and a member added and removed in
+ * one submit may be seen as an underflow.
  * A failure before the launch (descriptor upload) leaves every plane and N
  * as they were.  A failure of the launch itself (CPT_ECUDA) marks every plane
  * of the submit as failed: they may hold part of the ops, so submits and

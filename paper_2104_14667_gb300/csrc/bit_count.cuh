@@ -53,6 +53,16 @@ __device__ __forceinline__ void bitcount_add16(BitCounter &s, const uint32_t (&w
     }
 }
 
+// Sets the counts of the pixels whose bit is not in `mask` to zero.
+__device__ __forceinline__ void bitcount_keep(BitCounter &s, uint32_t mask) {
+    s.ones &= mask;
+    s.twos &= mask;
+    s.fours &= mask;
+    s.eights &= mask;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) s.hi[j] &= mask;
+}
+
 // The 32 counts of a BitCounter as 16 words of two 16-bit counts (pixel 2i in
 // the low half of pairs[i], pixel 2i+1 in the high half).  Eight pixels at a
 // time, byte b of each of the eight bit-slices becomes row j of an 8 x 8 bit
