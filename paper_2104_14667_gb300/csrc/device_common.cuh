@@ -149,6 +149,60 @@ __device__ __forceinline__ void atomic_count_group(CountT *dst, const uint32_t (
     if (under) flag_set(flags, kFlagUnderflow);
 }
 
+// One word of packed byte counters (four pixels) folded into dst, by a plain
+// read-modify-write or by atomics; as the group forms above.
+template <typename CountT>
+__device__ __forceinline__ void apply_count_word(CountT *dst, uint32_t packed, int sign, int *flags) {
+    bool under = false;
+    uint32_t c[4];
+    if constexpr (sizeof(CountT) == 2) {
+        const uint2 v = *reinterpret_cast<const uint2 *>(dst);
+        c[0] = v.x & 0xFFFFu, c[1] = v.x >> 16, c[2] = v.y & 0xFFFFu, c[3] = v.y >> 16;
+    } else {
+        const uint4 v = *reinterpret_cast<const uint4 *>(dst);
+        c[0] = v.x, c[1] = v.y, c[2] = v.z, c[3] = v.w;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const uint32_t d = (packed >> (8 * j)) & 0xFFu;
+        if (sign > 0) {
+            c[j] += d;
+        } else {
+            under |= d > c[j];
+            c[j] -= d;
+        }
+    }
+    if constexpr (sizeof(CountT) == 2)
+        *reinterpret_cast<uint2 *>(dst) = make_uint2((c[0] & 0xFFFFu) | (c[1] << 16), (c[2] & 0xFFFFu) | (c[3] << 16));
+    else
+        *reinterpret_cast<uint4 *>(dst) = make_uint4(c[0], c[1], c[2], c[3]);
+    if (under) flag_set(flags, kFlagUnderflow);
+}
+
+template <typename CountT>
+__device__ __forceinline__ void atomic_count_word(CountT *dst, uint32_t packed, int sign, int *flags) {
+    bool under = false;
+    constexpr int kPerWord = 4 / sizeof(CountT);   // counts in a 32-bit word of the plane
+#pragma unroll
+    for (int i = 0; i < 4 / kPerWord; ++i) {
+        uint32_t *w = reinterpret_cast<uint32_t *>(dst) + i;
+        const uint32_t dl = (packed >> (8 * kPerWord * i)) & 0xFFu;
+        const uint32_t dh = kPerWord == 2 ? (packed >> (16 * i + 8)) & 0xFFu : 0u;
+        const uint32_t d = dl | (dh << 16);
+        if (d == 0) continue;
+        if (sign > 0) {
+            atomicAdd(w, d);
+        } else {
+            const uint32_t old = atomicSub(w, d);
+            if constexpr (kPerWord == 2)
+                under |= (dl > (old & 0xFFFFu)) | (dh > (old >> 16));
+            else
+                under |= dl > old;
+        }
+    }
+    if (under) flag_set(flags, kFlagUnderflow);
+}
+
 // dst[j] (+|-)= acc[j] for the first `valid` of four float32 sums.
 __device__ __forceinline__ void apply_depth_group(float *dst, int valid, const float (&acc)[4],
                                                   int sign) {
