@@ -11,7 +11,7 @@
 // into the op's plane (uint32, or uint16 for a 16-bit plane): with L2
 // atomics, or with plain read-modify-writes when the plane's ops are single
 // slabs folded one after another by the same items (split_ops).  The render launch deals warp-level (plane,
-// chunk) items round robin to its warps.  Consecutive
+// 512 pixels) items round robin to its warps.  Consecutive
 // items are neighbouring chunks of the same slab, so concurrently running
 // warps read neighbouring bytes of the same members.
 #include <algorithm>
@@ -27,8 +27,7 @@
 #include "bit_count.cuh"
 #include "internal.cuh"
 #include "mask_load.cuh"
-#include "overlap_class.cuh"
-#include "class_histogram.cuh"
+#include "render_units.cuh"
 
 namespace {
 
@@ -65,20 +64,19 @@ struct OpDesc {
     int32_t chain;               // ops folded by this op's items: itself and the chain - 1 that follow it
 };
 
-// One render op.  The plane's pitch is groups_per_row x 16 pixels, so group g of the plane holds
-// the counts of pixels 16 g .. 16 g + 15 in memory order.
+// One render op: its output pixels in items of 512 (render_units.cuh).
 struct RenderDesc {
-    const uint32_t *plane;
+    const void *plane;
     void *counts_out;
     uint8_t *bucket_out;
     uint32_t *rgba_out;
     int64_t item_start;
+    int64_t pitch;         // of the plane, elements
+    int64_t pixels;
     int32_t width;
-    int32_t height;
-    int32_t groups_per_row;
-    int32_t vec;           // 16-byte stores allowed
+    int32_t rows;          // cpt::PlaneRows
+    int32_t vec;           // outputs aligned to four of their elements
     int32_t u16;           // the plane holds uint16 counts (else uint32)
-    int32_t dense;         // width == plane pitch: group g's outputs start at 16 g
     cpt::ClassDivisor div; // floor(255 c / n_members) by multiplication
     unsigned long long *hist;   // 256 class counts, zeroed before the launch, or NULL
 };
@@ -152,14 +150,18 @@ __device__ __forceinline__ void load_starts(const Desc *d, int n, uint32_t *star
 template <bool kGather>
 __device__ __forceinline__ void fold_group(const uint8_t *row, int64_t stride, int m0, const int32_t *index, int cnt,
                                            int exact, uint32_t (&k)[4]) {
-    const uint8_t *q = kGather ? row : row + (int64_t)m0 * stride;
-    auto at = [&](int i) { return kGather ? q + (int64_t)index[i] * stride : q + (int64_t)i * stride; };
-    if (exact == 0) {
+    if (exact != 0) {
+#pragma unroll 4
+        for (int i = 0; i < cnt; ++i)
+            cpt::add_group(k, cpt::load_group_exact(row + (int64_t)(kGather ? index[i] : m0 + i) * stride, exact));
+    } else if (!kGather) {
+        cpt::fold_masks<true>(row, stride, m0, m0 + cnt, k);
+    } else {
         int i = 0;
         for (; i + 8 <= cnt; i += 8) {
             uint4 v[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = __ldcs(reinterpret_cast<const uint4 *>(at(i + j)));
+            for (int j = 0; j < 8; ++j) v[j] = __ldcs(reinterpret_cast<const uint4 *>(row + (int64_t)index[i + j] * stride));
 #pragma unroll
             for (int j = 0; j < 8; ++j) cpt::add_group(k, v[j]);
         }
@@ -168,14 +170,11 @@ __device__ __forceinline__ void fold_group(const uint8_t *row, int64_t stride, i
 #pragma unroll
             for (int j = 0; j < 7; ++j) {
                 v[j] = make_uint4(0u, 0u, 0u, 0u);
-                if (i + j < cnt) v[j] = __ldcs(reinterpret_cast<const uint4 *>(at(i + j)));
+                if (i + j < cnt) v[j] = __ldcs(reinterpret_cast<const uint4 *>(row + (int64_t)index[i + j] * stride));
             }
 #pragma unroll
             for (int j = 0; j < 7; ++j) cpt::add_group(k, v[j]);
         }
-    } else {
-#pragma unroll 4
-        for (int i = 0; i < cnt; ++i) cpt::add_group(k, cpt::load_group_exact(at(i), exact));
     }
 }
 
@@ -393,62 +392,61 @@ engine_clear_kernel(const ClearDesc *ops, int n_ops, uint32_t n_items, int *flag
     }
 }
 
-// Classify and store one lane's group of 16 pixels (counts c, as loaded in
-// v); row: the lane's histogram counters, or NULL.
-template <bool kHist, bool kNarrow>
-__device__ __forceinline__ void render_group(const RenderDesc &op, const uint4 (&v)[4], const uint32_t (&c)[16], int valid,
-                                             int64_t out, int pieces, const uint32_t *table, uint8_t *row,
-                                             uint32_t key) {
-    auto cls = [&](uint32_t x) {
-        return kNarrow ? cpt::overlap_class_narrow(x, op.div) : cpt::overlap_class(x, op.div);
-    };
-    if (op.vec && valid == 16) {
-        if (op.counts_out) {
+// One warp item of a render op: every lane loads its units' counts, `between`
+// runs while they are on their way, then the units are classified and stored.
+// row: the lane's histogram counters, or NULL.  The row form and the class
+// path (one multiply-high below 2^16 members, the general division above) are
+// chosen per item, so that each keeps only its own values live.
+template <typename CountT, bool kNarrow>
+__device__ __forceinline__ void store_item(const RenderDesc &op, const cpt::Unit<CountT> (&c)[cpt::kUnits], int64_t base,
+                                           int left, int lane, const uint32_t *table, uint8_t *row, uint32_t key) {
+    CountT *counts_out = static_cast<CountT *>(op.counts_out);
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (q < pieces)   // 'pieces' bytes per count
-                    reinterpret_cast<uint4 *>(static_cast<uint8_t *>(op.counts_out) + out * pieces)[q] = v[q];
-        }
-        // a quarter of the group at a time: classes, their colours, the packed classes
-        uint32_t w[4];
+    for (int k = 0; k < cpt::kUnits; ++k) {
+        const int at = 4 * (32 * k + lane);
+        if (at >= left) break;
+        uint32_t b[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t b0 = cls(c[4 * q]), b1 = cls(c[4 * q + 1]);
-            const uint32_t b2 = cls(c[4 * q + 2]), b3 = cls(c[4 * q + 3]);
-            w[q] = b0 | (b1 << 8) | (b2 << 16) | (b3 << 24);
-            if (kHist && row) cpt::hist_count_quarter(row, key, b0, b1, b2, b3);
-            if (op.rgba_out)
-                reinterpret_cast<uint4 *>(op.rgba_out + out)[q] = make_uint4(table[b0], table[b1], table[b2], table[b3]);
-        }
-        if (op.bucket_out) *reinterpret_cast<uint4 *>(op.bucket_out + out) = make_uint4(w[0], w[1], w[2], w[3]);
-    } else {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            if (j < valid) {
-                const uint32_t b = cls(c[j]);
-                if (op.counts_out) {
-                    if (op.u16)
-                        reinterpret_cast<uint16_t *>(op.counts_out)[out + j] = (uint16_t)c[j];
-                    else
-                        reinterpret_cast<uint32_t *>(op.counts_out)[out + j] = c[j];
-                }
-                if (op.bucket_out) op.bucket_out[out + j] = (uint8_t)b;
-                if (op.rgba_out) op.rgba_out[out + j] = table[b];
-                if (kHist && row) cpt::hist_add(row, key, b, 1u);
-            }
-        }
+        for (int j = 0; j < 4; ++j)
+            b[j] = kNarrow ? cpt::overlap_class_narrow(c[k].get(j), op.div) : cpt::overlap_class(c[k].get(j), op.div);
+        cpt::store_unit(c[k], b, base + at, left - at, op.vec != 0, counts_out, op.bucket_out, op.rgba_out, table, row, key);
     }
 }
 
-// Render: warp-level items (render op, 32 16-pixel groups of its plane, one
-// per lane) dealt round robin to every warp of the launch -- items are all
-// the same size, so no counter is needed.  With histograms (kHist; 5 KB of
-// dynamic shared memory per warp) every CTA takes one contiguous range of
-// items instead, so that a warp's items span one or two ops and its totals
-// go to global memory once or twice.  A plane's pitch is a whole number of
-// groups, so group g holds the counts of pixels 16 g .. 16 g + 15 in memory
-// order; when the outputs are dense at that pitch too (width a multiple of
-// 16) they start at 16 g as well and no row division is needed.
+template <typename CountT, int kRows>
+__device__ __forceinline__ void load_item(const RenderDesc &op, int64_t base, int left, int lane,
+                                          cpt::Unit<CountT> (&c)[cpt::kUnits]) {
+    const CountT *plane = static_cast<const CountT *>(op.plane);
+#pragma unroll
+    for (int k = 0; k < cpt::kUnits; ++k) {
+        const int at = 4 * (32 * k + lane);
+        if (at < left) cpt::load_unit<CountT, kRows>(plane, op.pitch, op.width, base + at, left - at, c[k]);
+    }
+}
+
+template <typename CountT, typename Between>
+__device__ __forceinline__ void render_item(const RenderDesc &op, int64_t base, int lane, const uint32_t *table, uint8_t *row,
+                                            uint32_t key, Between between) {
+    const int left = (int)min(op.pixels - base, (int64_t)cpt::kItemPixels);
+    cpt::Unit<CountT> c[cpt::kUnits];
+    if (op.rows == cpt::kRowsDense)
+        load_item<CountT, cpt::kRowsDense>(op, base, left, lane, c);
+    else if (op.rows == cpt::kRowsOfFours)
+        load_item<CountT, cpt::kRowsOfFours>(op, base, left, lane, c);
+    else
+        load_item<CountT, cpt::kRowsRagged>(op, base, left, lane, c);
+    between();
+    if (op.div.narrow)
+        store_item<CountT, true>(op, c, base, left, lane, table, row, key);
+    else
+        store_item<CountT, false>(op, c, base, left, lane, table, row, key);
+}
+
+// Render: warp-level items (render op, 512 of its pixels) dealt round robin
+// to every warp of the launch -- items are all the same size, so no counter is
+// needed.  With histograms (kHist; 5 KB of dynamic shared memory per warp)
+// every CTA takes one contiguous range of items instead, so that a warp's
+// items span one or two ops and its totals go to global memory once or twice.
 template <bool kHist>
 __global__ void __launch_bounds__(kThreads, kHist ? kRenderHistCtasPerSm : kRenderCtasPerSm)
 engine_render_kernel(const RenderDesc *__restrict__ ops, int n_ops, uint32_t n_items, Lut lut) {
@@ -506,49 +504,19 @@ engine_render_kernel(const RenderDesc *__restrict__ ops, int n_ops, uint32_t n_i
             }
             ++since_fold;
         }
-        const int64_t groups = (int64_t)op.groups_per_row * op.height;
-        const int64_t g = (int64_t)(item - (uint32_t)op.item_start) * 32 + lane;
-        const int pieces = op.u16 ? 2 : 4;   // 16-byte pieces of a group's counts
-        const uint4 *src = reinterpret_cast<const uint4 *>(op.plane) + g * pieces;
-        uint4 v[4];
-        if (g < groups) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (q < pieces) v[q] = src[q];
-        }
+        const int64_t base = (int64_t)(item - (uint32_t)op.item_start) * cpt::kItemPixels;
         const uint32_t next = item + stride;
-        if (!kHist && next < last && idx + 1 < n_ops && next >= op_start(ops, n_ops, s_starts, idx + 1))
-            idx = find_op(ops, n_ops, s_starts, next);
-        if (g >= groups) continue;
-        uint32_t c[16];
-        if (op.u16) {
-            const uint32_t w[8] = {v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w};
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                c[2 * q] = w[q] & 0xFFFFu;
-                c[2 * q + 1] = w[q] >> 16;
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                c[4 * q] = v[q].x; c[4 * q + 1] = v[q].y; c[4 * q + 2] = v[q].z; c[4 * q + 3] = v[q].w;
-            }
-        }
-        int valid = 16;
-        int64_t out = g * 16;
-        if (!op.dense) {
-            const int y = (int)(g / op.groups_per_row);
-            const int x0 = (int)(g - (int64_t)y * op.groups_per_row) * 16;
-            valid = min(16, op.width - x0);
-            out = (int64_t)y * op.width + x0;
-        }
-        // one multiply-high per class for N < 2^16 (every 16-bit plane), the
-        // general division otherwise: a branch per item, so that each
-        // specialisation keeps only its own divisor fields live
-        if (op.div.narrow)
-            render_group<kHist, true>(op, v, c, valid, out, pieces, table, hist_at ? row : nullptr, key);
+        int next_idx = idx;
+        auto look_up = [&]() {
+            if (!kHist && next < last && idx + 1 < n_ops && next >= op_start(ops, n_ops, s_starts, idx + 1))
+                next_idx = find_op(ops, n_ops, s_starts, next);
+        };
+        uint8_t *count_into = kHist && hist_at ? row : nullptr;
+        if (op.u16)
+            render_item<uint16_t>(op, base, lane, table, count_into, key, look_up);
         else
-            render_group<kHist, false>(op, v, c, valid, out, pieces, table, hist_at ? row : nullptr, key);
+            render_item<uint32_t>(op, base, lane, table, count_into, key, look_up);
+        idx = next_idx;
     }
     if (kHist && hist_at) {
         cpt::hist_fold(cnt, tot, lane);
@@ -947,17 +915,15 @@ int plan_render(composite_engine *e, const composite_render_op *ops, int32_t n_o
         d.rgba_out = reinterpret_cast<uint32_t *>(o.rgba_out);
         d.item_start = items;
         d.div = cpt::class_divisor((uint64_t)n);
+        d.pitch = p.pitch_px;
+        d.pixels = (int64_t)p.width * p.height;
         d.width = p.width;
-        d.height = p.height;
-        d.groups_per_row = (int32_t)(p.pitch_px / 16);
-        const int64_t groups = (int64_t)d.groups_per_row * p.height;
-        const int64_t tiles = (groups + 31) / 32;   // warp items: one 16-pixel group per lane
-        const uintptr_t a = reinterpret_cast<uintptr_t>(o.counts_out) | reinterpret_cast<uintptr_t>(o.bucket_out) |
-                            reinterpret_cast<uintptr_t>(o.rgba_out);
-        d.vec = (p.width % 16 == 0) && (a % 16 == 0);
+        d.rows = cpt::plane_rows(p.pitch_px, p.width);
+        d.vec = reinterpret_cast<uintptr_t>(o.counts_out) % (4 * (p.count_bits / 8)) == 0 &&
+                reinterpret_cast<uintptr_t>(o.bucket_out) % 4 == 0 && reinterpret_cast<uintptr_t>(o.rgba_out) % 16 == 0;
         d.u16 = p.count_bits == 16 ? 1 : 0;
-        d.dense = p.pitch_px == p.width ? 1 : 0;
         d.hist = reinterpret_cast<unsigned long long *>(o.histogram_out);
+        const int64_t tiles = (d.pixels + cpt::kItemPixels - 1) / cpt::kItemPixels;
         items += tiles;
         descs->push_back(d);
     }
