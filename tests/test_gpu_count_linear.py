@@ -60,6 +60,32 @@ def test_depths_at_any_alignment(w, h, shift, pad, gap):
             assert err <= 4.0 * n * 2.0 ** -24
 
 
+@pytest.mark.parametrize("w,h,shift", [(64, 8, 0), (61, 9, 3)])
+def test_depth_sums_of_many_members_round_seldom(w, h, shift):
+    n = 1000
+    d = synth.random_depths(5, n, h, w)
+    with binding.Composite(w, h, mode="mean_depth") as comp:
+        comp.add(shifted(d, shift, w, 0))
+        err = np.abs(comp.render_host()["mean"].astype(np.float64) - oracle.mean_depth(d)).max()
+    # a value of at most 4 n meets 3 roundings in a tree of 8, 8 in a block, 16 blocks, 3 slices, and the division
+    assert err <= 4.0 * (3 + 8 + 16 + 3 + 1) * 2.0 ** -24
+
+
+@pytest.mark.parametrize("count_bits", [16, 32])
+@pytest.mark.parametrize("w,h,shift,pad,gap", LAYOUTS + [(8, 4, 3, 1, 0), (33, 3, 4, 3, 4), (200, 9, 8, 7, 8), (1856, 5, 0, 0, 0)])
+def test_bit_rows_at_any_alignment(w, h, shift, pad, gap, count_bits):
+    with binding.Composite(w, h, count_bits=count_bits, mask_format="bits") as comp:
+        for n in MEMBERS:
+            m = synth.random_masks(n, n, h, w)
+            packed = synth.pack_masks(m)
+            dev = shifted(packed, shift, packed.shape[2] + pad, gap)
+            comp.clear()
+            comp.add(dev)
+            np.testing.assert_array_equal(comp.render_host()["counts"].astype(np.int64), oracle.count(m))
+            comp.remove(dev[: n // 2])
+            np.testing.assert_array_equal(comp.render_host()["counts"].astype(np.int64), oracle.count(m[n // 2:]))
+
+
 def test_more_members_than_the_slabs_of_one_launch():
     n, limit = 65535 * 255 + 300, 65535 * 255
     base = torch.zeros((n, 1, 1), dtype=torch.uint8, device="cuda")
