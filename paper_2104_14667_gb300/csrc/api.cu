@@ -696,9 +696,9 @@ int apply(composite_ctx *ctx, const void *members, int32_t n, int64_t stride, in
             const bool direct = (ctx->width % ctx->vec_px == 0) && stride == (int64_t)pitch * ctx->height;
             rc = direct ? run_texture_from_device(ctx, src, n, stride, pitch, sign)
                         : run_staged(ctx, src, n, stride, pitch, sign);
-        } else if (aligned || (ctx->cfg.read_path == CPT_READ_LINEAR && !ctx->bits)) {
+        } else if (aligned || ctx->cfg.read_path == CPT_READ_LINEAR) {
             // read in place: the linear kernels take any alignment, the tensor
-            // map and the bit kernels 16 bytes
+            // map 16 bytes
             RasterBatch b{members, stride, pitch, n};
             rc = begin_chunk(ctx);
             if (!rc) rc = accumulate(ctx, b, sign);

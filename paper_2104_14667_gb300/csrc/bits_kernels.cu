@@ -4,6 +4,7 @@
 #include <algorithm>
 
 #include "bit_count.cuh"
+#include "mask_load.cuh"
 
 namespace cpt {
 namespace {
@@ -11,19 +12,33 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kPackedLimit = 255;   // members a bit-sliced counter can hold
 
+// How a lane reads its share of a member's row.
+enum WordLoads {
+    kPairs = 0,     // two words, rows 8-byte aligned: a warp reads 256 contiguous bytes per member
+    kSingles = 1,   // one word, rows 4-byte aligned
+    kShifted = 2    // one word at any byte address, cut out of the two aligned words that hold it
+};
+
 // Bit-packed masks (one bit per pixel, pixel x at bit x & 7 of byte x >> 3 of
-// the row).  A thread owns kWords 32-pixel words of a composite row (with
-// kWords = 2 a warp reads 256 contiguous bytes per member, 8 per lane) and
+// the row).  A thread owns one or two 32-pixel words of a composite row and
 // keeps the slab's counts in BitCounters (carry-save accumulators, see
-// bit_count.cuh); whole steps of 16 members load without predicates, and
-// the counts leave the bit-sliced form through bitcount_pairs.
-template <typename CountT, int kWords>
+// bit_count.cuh), 16 members per step; the bits past a row's last pixel are
+// counted along (they are row padding, or the next row's) and dropped from
+// the counters at the end, and the counts leave the bit-sliced form through
+// bitcount_pairs.  Bound by memory latency: the bytes in flight wait in
+// registers.  Rows that are no multiple of 16 bytes used to be copied into
+// staging slots first: 1856 x 2208 x 1024 (rows of 232 bytes, which the
+// bulk-copy kernel now takes in place) 852 us with clear and render.
+template <typename CountT, int kLoads>
 __global__ void __launch_bounds__(kThreads, 4)
 count_bits_kernel(RasterBatch b, Plane p, int sign, int *flags, int64_t units, int units_per_row,
                   int slab, int slabs) {
+    constexpr int kWords = kLoads == kPairs ? 2 : 1;
     constexpr int kPix = 32 * kWords;
     CountT *plane = static_cast<CountT *>(p.data);
     const int64_t stride = b.member_stride;
+    const uint8_t *base = static_cast<const uint8_t *>(b.base);
+    const uint8_t *end = batch_end(b, (p.width + 7) / 8, p.height);
     for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < units * slabs;
          u += (int64_t)gridDim.x * blockDim.x) {
         const int sl = (int)(u / units);
@@ -34,71 +49,80 @@ count_bits_kernel(RasterBatch b, Plane p, int sign, int *flags, int64_t units, i
         const int valid = min(kPix, p.width - x0);
         const int m0 = sl * slab;
         const int m1 = min(b.n, m0 + slab);
-        const uint8_t *q = static_cast<const uint8_t *>(b.base) + (int64_t)y * b.row_pitch + gx * 4 * kWords +
-                           (int64_t)m0 * stride;
+        const uint8_t *at = base + (int64_t)y * b.row_pitch + gx * 4 * kWords;
+        int f0, f1;
+        safe_members(at, stride, base, end, 4 * kWords, kLoads == kSingles ? 4 : 8, m0, m1, f0, f1);
         BitCounter acc[kWords];
-        int m = m0;
-        if (valid == kPix) {
-            for (; m + 16 <= m1; m += 16) {
-                uint32_t w[kWords][16];
+        const uint8_t *q = at + (int64_t)f0 * stride;
+        for (int left = f1 - f0; left > 0; left -= 16) {
+            uint32_t w[kWords][16], hi[16], shift[16];
 #pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    if constexpr (kWords == 2) {
-                        const uint2 v = __ldcs(reinterpret_cast<const uint2 *>(q + k * stride));
-                        w[0][k] = v.x;
-                        w[1][k] = v.y;
-                    } else {
-                        w[0][k] = __ldcs(reinterpret_cast<const uint32_t *>(q + k * stride));
-                    }
+            for (int k = 0; k < 16; ++k, q += stride) {
+                const uint8_t *r = q;
+                if constexpr (kLoads == kPairs) {
+                    uint2 v = make_uint2(0u, 0u);
+                    if (k < left) v = __ldcs(reinterpret_cast<const uint2 *>(r));
+                    w[0][k] = v.x;
+                    w[1][k] = v.y;
+                } else if constexpr (kLoads == kSingles) {
+                    w[0][k] = k < left ? __ldcs(reinterpret_cast<const uint32_t *>(r)) : 0u;
+                } else {
+                    shift[k] = (uint32_t)reinterpret_cast<uintptr_t>(r) & 3u;
+                    const uint32_t *block = reinterpret_cast<const uint32_t *>(r - shift[k]);
+                    w[0][k] = k < left ? __ldg(block) : 0u;
+                    hi[k] = k < left ? __ldg(block + 1) : 0u;
                 }
-#pragma unroll
-                for (int j = 0; j < kWords; ++j) bitcount_add16(acc[j], w[j]);
-                q += 16 * stride;
             }
+            if constexpr (kLoads == kShifted)
+#pragma unroll
+                for (int k = 0; k < 16; ++k) w[0][k] = __funnelshift_r(w[0][k], hi[k], 8u * shift[k]);
+#pragma unroll
+            for (int j = 0; j < kWords; ++j) bitcount_add16(acc[j], w[j]);
         }
-        // the slab's last (< 16) members, and every member at a ragged right
-        // edge: word by word, bits past the width dropped
-        for (; m < m1; m += 16) {
-            const int take = min(16, m1 - m);
+        // the few members whose aligned loads would leave the batch, byte by byte
+        auto exact = [&](int m) {
+            const uint8_t *r = at + (int64_t)m * stride;
+            const int nbytes = (valid + 7) / 8;
 #pragma unroll
             for (int j = 0; j < kWords; ++j) {
-                const int vj = min(32, max(0, valid - 32 * j));
-                const int nbytes = (vj + 7) / 8;
-                const uint32_t keep = vj == 32 ? 0xFFFFFFFFu : ((1u << vj) - 1u);
-                uint32_t w[16];
+                uint32_t w[16] = {0u};
 #pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    uint32_t v = 0;
-                    if (k < take) {
-                        const uint8_t *r = q + k * stride + 4 * j;
-                        if (vj == 32)
-                            v = __ldcs(reinterpret_cast<const uint32_t *>(r));
-                        else
-                            for (int i = 0; i < nbytes; ++i) v |= (uint32_t)r[i] << (8 * i);
-                    }
-                    w[k] = v & keep;
-                }
+                for (int i = 0; i < 4; ++i)
+                    if (4 * j + i < nbytes) w[0] |= (uint32_t)r[4 * j + i] << (8 * i);
                 bitcount_add16(acc[j], w);
             }
-            q += 16 * stride;
-        }
+        };
+        for (int m = m0; m < f0; ++m) exact(m);
+        for (int m = f1; m < m1; ++m) exact(m);
         CountT *dst = plane + (int64_t)y * p.pitch + x0;
 #pragma unroll
         for (int j = 0; j < kWords; ++j) {
-            if (valid <= 32 * j) break;
+            const int vj = valid - 32 * j;
+            if (vj <= 0) break;
+            if (vj < 32) bitcount_keep(acc[j], (1u << vj) - 1u);
             uint32_t pairs[16];
             bitcount_pairs(acc[j], pairs);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {           // two 16-pixel groups per word
-                const int v = min(16, valid - 32 * j - 16 * h);
-                if (v <= 0) break;
+                if (vj <= 16 * h) break;            // a half word past the plane's pitch
                 if (slabs == 1)
-                    apply_pair_group<CountT>(dst + 32 * j + 16 * h, v, pairs + 8 * h, sign, flags);
+                    apply_pair_group<CountT>(dst + 32 * j + 16 * h, 16, pairs + 8 * h, sign, flags);
                 else
                     atomic_pair_group<CountT>(dst + 32 * j + 16 * h, pairs + 8 * h, sign, flags);
             }
         }
     }
+}
+
+template <typename CountT>
+void launch_count_bits_t(int loads, unsigned grid, cudaStream_t s, const RasterBatch &b, const Plane &p, int sign, int *flags,
+                         int64_t units, int per_row, int slab, int slabs) {
+    if (loads == kPairs)
+        count_bits_kernel<CountT, kPairs><<<grid, kThreads, 0, s>>>(b, p, sign, flags, units, per_row, slab, slabs);
+    else if (loads == kSingles)
+        count_bits_kernel<CountT, kSingles><<<grid, kThreads, 0, s>>>(b, p, sign, flags, units, per_row, slab, slabs);
+    else
+        count_bits_kernel<CountT, kShifted><<<grid, kThreads, 0, s>>>(b, p, sign, flags, units, per_row, slab, slabs);
 }
 
 inline int64_t blocks_for(int64_t groups) {
@@ -113,9 +137,9 @@ cudaError_t launch_count_bits(const RasterBatch &b, const Plane &p, int sign, in
     const int wpr = (p.width + 31) / 32;
     if (b.n <= 0 || wpr == 0 || p.height == 0) return cudaSuccess;
     // two words (8 bytes) per thread and member where every row start is 8-byte aligned
-    const bool wide = wpr >= 2 && reinterpret_cast<uintptr_t>(b.base) % 8 == 0 && b.row_pitch % 8 == 0 &&
-                      b.member_stride % 8 == 0;
-    const int per_row = wide ? (wpr + 1) / 2 : wpr;
+    const uint64_t places = reinterpret_cast<uintptr_t>(b.base) | (uint64_t)b.row_pitch | (uint64_t)b.member_stride;
+    const int loads = wpr >= 2 && places % 8 == 0 ? kPairs : places % 4 == 0 ? kSingles : kShifted;
+    const int per_row = loads == kPairs ? (wpr + 1) / 2 : wpr;
     const int64_t units = (int64_t)per_row * p.height;
     // member slabs of at most 255 (eight counter levels); more only to fill
     // about four waves of four 256-thread CTAs per SM, since every slab pays
@@ -127,17 +151,10 @@ cudaError_t launch_count_bits(const RasterBatch &b, const Plane &p, int sign, in
     const int slab = (int)((b.n + slabs - 1) / slabs);
     slabs = (b.n + slab - 1) / slab;
     const unsigned grid = (unsigned)blocks_for(units * slabs);
-    if (p.count_bits == 16) {
-        if (wide)
-            count_bits_kernel<uint16_t, 2><<<grid, kThreads, 0, s>>>(b, p, sign, flags, units, per_row, slab, (int)slabs);
-        else
-            count_bits_kernel<uint16_t, 1><<<grid, kThreads, 0, s>>>(b, p, sign, flags, units, per_row, slab, (int)slabs);
-    } else {
-        if (wide)
-            count_bits_kernel<uint32_t, 2><<<grid, kThreads, 0, s>>>(b, p, sign, flags, units, per_row, slab, (int)slabs);
-        else
-            count_bits_kernel<uint32_t, 1><<<grid, kThreads, 0, s>>>(b, p, sign, flags, units, per_row, slab, (int)slabs);
-    }
+    if (p.count_bits == 16)
+        launch_count_bits_t<uint16_t>(loads, grid, s, b, p, sign, flags, units, per_row, slab, (int)slabs);
+    else
+        launch_count_bits_t<uint32_t>(loads, grid, s, b, p, sign, flags, units, per_row, slab, (int)slabs);
     return cudaGetLastError();
 }
 
