@@ -79,8 +79,10 @@ enum {
 /* The buffer-to-image transform of the texture path (Section 4). */
 enum {
     CPT_CONVERT_COPY = 0,     /* cudaMemcpy3DAsync into the array (the driver's copy)      */
-    CPT_CONVERT_KERNEL = 1    /* a kernel: 16-byte loads, surface stores into the array;
-                                 unaligned sources fall back to the copy                */
+    CPT_CONVERT_KERNEL = 1    /* a kernel: 16-byte loads, surface stores into the array.
+                                 Masks become one bit per pixel there, from rasters of
+                                 any layout; depths keep their bytes, and unaligned
+                                 depths fall back to the copy                           */
 };
 
 /* How pageable host rasters reach the device (step a2). */

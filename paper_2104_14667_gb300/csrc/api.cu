@@ -72,6 +72,8 @@ struct composite_ctx {
     int slot_members = 0;      // rasters a staging slot holds: chunk_members, or the automatic depth's cap
     int call_chunk = 0;        // C of the current add/remove
     bool bits = false;         // masks are bit-packed
+    bool packed_array = false; // texture path: the arrays hold one bit per pixel
+    int array_layers = 0;      // texture path: layers of a slot's array
     Plane plane{};
     int *flags = nullptr;      // device flags
     int *h_flags = nullptr;    // pinned copy of the flags
@@ -334,6 +336,13 @@ int setup(composite_ctx *ctx) {
         if (groups > maxw || ctx->height > maxh || ctx->slot_members > maxl)
             return fail(ctx, CPT_EINVAL, "raster %dx%d with %d layers exceeds the layered texture limits (%d texels, %d rows, %d layers)",
                         ctx->width, ctx->height, ctx->slot_members, maxw, maxh, maxl);
+        // Masks that the library's kernel converts become one bit per pixel:
+        // with the automatic depth an array then holds eight slots' worth of
+        // layers in the bytes that one slot of byte masks takes.
+        ctx->packed_array = c.mode == CPT_MODE_COUNT && c.layout_converter == CPT_CONVERT_KERNEL;
+        ctx->array_layers = ctx->slot_members;
+        if (ctx->packed_array && c.chunk_members == 0)
+            ctx->array_layers = std::min(std::min(255, maxl), 8 * ctx->slot_members);
     }
 
     const int count_bytes = c.mode == CPT_MODE_COUNT ? c.count_bits / 8 : 4;
@@ -356,11 +365,12 @@ int setup(composite_ctx *ctx) {
         CK(ctx, cudaEventCreateWithFlags(&s.ring_free, cudaEventDisableTiming));
         if (c.read_path == CPT_READ_TEXTURE) {
             cudaChannelFormatDesc desc =
-                c.mode == CPT_MODE_COUNT
+                ctx->packed_array ? cudaCreateChannelDesc(32, 32, 0, 0, cudaChannelFormatKindUnsigned)
+                : c.mode == CPT_MODE_COUNT
                     ? cudaCreateChannelDesc(32, 32, 32, 32, cudaChannelFormatKindUnsigned)
                     : cudaCreateChannelDesc(32, 32, 32, 32, cudaChannelFormatKindFloat);
-            CK(ctx, cudaMalloc3DArray(&s.array, &desc,
-                                      make_cudaExtent((size_t)groups, ctx->height, ctx->slot_members),
+            const size_t texels = ctx->packed_array ? (size_t)cpt::packed_texels(ctx->width) : (size_t)groups;
+            CK(ctx, cudaMalloc3DArray(&s.array, &desc, make_cudaExtent(texels, ctx->height, ctx->array_layers),
                                       cudaArrayLayered | cudaArraySurfaceLoadStore));
             cudaResourceDesc rd{};
             rd.resType = cudaResourceTypeArray;
@@ -420,20 +430,30 @@ int accumulate_texture(composite_ctx *ctx, Slot &s, int n_layers, int sign) {
     int rc = trace_open(ctx, kTraceKernel, ctx->compute);
     if (rc) return rc;
     const cudaError_t e =
-        ctx->cfg.mode == CPT_MODE_COUNT
+        ctx->packed_array
+            ? cpt::launch_count_packed_texture(s.tex, n_layers, ctx->plane, sign, ctx->flags, ctx->caps, ctx->compute)
+        : ctx->cfg.mode == CPT_MODE_COUNT
             ? cpt::launch_count_texture(s.tex, n_layers, ctx->plane, sign, ctx->flags, ctx->caps, ctx->compute)
             : cpt::launch_depth_texture(s.tex, n_layers, ctx->plane, sign, ctx->flags, ctx->caps, ctx->compute);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "texture kernel launch");
     return trace_close(ctx, ctx->compute);
 }
 
-// Layout conversion into the slot's cudaArray (the buffer-to-image copy of
-// Section 4), from `src` rasters with row pitch `pitch` and raster stride
-// pitch * height, on stream st.
-int convert_to_array(composite_ctx *ctx, Slot &s, const void *src, int64_t pitch, int n_layers,
-                     cudaStream_t st) {
+// Layout conversion into the first layers of the slot's cudaArray (the
+// buffer-to-image copy of Section 4) on stream st.  Arrays of bits take
+// rasters of any layout; byte and float arrays rasters whose stride is
+// pitch * height.
+int convert_to_array(composite_ctx *ctx, Slot &s, const RasterBatch &b, cudaStream_t st) {
     int rc = trace_open(ctx, kTraceConvert, st);
     if (rc) return rc;
+    if (ctx->packed_array) {
+        const cudaError_t e = cpt::launch_pack_to_array(b, ctx->width, ctx->height, s.surf, st);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "layout conversion kernel launch");
+        return trace_close(ctx, st);
+    }
+    const void *src = b.base;
+    const int64_t pitch = b.row_pitch;
+    const int n_layers = b.n;
     const int texels = (int)(ctx->pitch_px / ctx->vec_px);
     const bool aligned = (reinterpret_cast<uintptr_t>(src) % 16 == 0) && (pitch % 16 == 0);
     if (ctx->cfg.layout_converter == CPT_CONVERT_KERNEL && aligned) {
@@ -453,12 +473,12 @@ int convert_to_array(composite_ctx *ctx, Slot &s, const void *src, int64_t pitch
 
 // Consumes one staged chunk on the compute stream.
 int consume_slot(composite_ctx *ctx, Slot &s, int c, int sign) {
+    RasterBatch b{s.stage, ctx->member_bytes, ctx->stage_pitch, c};
     if (ctx->cfg.read_path == CPT_READ_TEXTURE) {
-        int rc = convert_to_array(ctx, s, s.stage, ctx->stage_pitch, c, ctx->compute);
+        int rc = convert_to_array(ctx, s, b, ctx->compute);
         if (rc) return rc;
         return accumulate_texture(ctx, s, c, sign);
     }
-    RasterBatch b{s.stage, ctx->member_bytes, ctx->stage_pitch, c};
     return accumulate(ctx, b, sign);
 }
 
@@ -511,23 +531,40 @@ int run_staged(composite_ctx *ctx, const uint8_t *src, int n, int64_t stride, in
 }
 
 // Device rasters on the texture path, converted straight from the caller's
-// memory into the slot arrays on the copy stream.
+// memory into the slot arrays on the copy stream.  Into an array of bits go as
+// many chunks at a time as it has layers for, by one conversion and one fold
+// (8 members of 2048^2 at a time were 32 short launches of each, and waits of
+// one stream for the other); the first of the chunks gets a trace record of
+// the conversion's interval, the others empty ones at its end.
 int run_texture_from_device(composite_ctx *ctx, const uint8_t *src, int n, int64_t stride, int64_t pitch, int sign) {
     const int C = ctx->call_chunk;
-    for (int m0 = 0; m0 < n; m0 += C) {
+    int per_array = ctx->packed_array ? std::max(C, ctx->array_layers / C * C) : C;
+    // in equal parts, whole chunks each: a short last one would be a conversion and a fold for little
+    const int arrays = (n + per_array - 1) / per_array;
+    per_array = std::min(per_array, ((n + arrays - 1) / arrays + C - 1) / C * C);
+    for (int a0 = 0; a0 < n; a0 += per_array) {
         const cpt::TraceRange chunk_range("composite chunk");
-        const int c = n - m0 < C ? n - m0 : C;
-        int rc = begin_chunk(ctx);
-        if (rc) return rc;
-        Slot &s = next_slot(ctx);
-        CK(ctx, cudaStreamWaitEvent(ctx->copy, s.consumed, 0));
-        rc = convert_to_array(ctx, s, src + (int64_t)m0 * stride, pitch, c, ctx->copy);
-        if (rc) return rc;
-        CK(ctx, cudaEventRecord(s.ready, ctx->copy));
-        CK(ctx, cudaStreamWaitEvent(ctx->compute, s.ready, 0));
-        rc = accumulate_texture(ctx, s, c, sign);
-        if (rc) return rc;
-        CK(ctx, cudaEventRecord(s.consumed, ctx->compute));
+        int take = 0, chunks = 0, refused = CPT_OK;
+        while (take < per_array && a0 + take < n && !(refused = begin_chunk(ctx))) {
+            take = std::min(std::min(take + C, per_array), n - a0);
+            ++chunks;
+        }
+        if (take > 0) {
+            Slot &s = next_slot(ctx);
+            CK(ctx, cudaStreamWaitEvent(ctx->copy, s.consumed, 0));
+            int rc = convert_to_array(ctx, s, RasterBatch{src + (int64_t)a0 * stride, stride, pitch, take}, ctx->copy);
+            if (rc) return rc;
+            if (ctx->cfg.trace) {
+                const cudaEvent_t end = ctx->trace.back().b;
+                ctx->trace.insert(ctx->trace.end(), chunks - 1, TraceRec{kTraceConvert, end, end});
+            }
+            CK(ctx, cudaEventRecord(s.ready, ctx->copy));
+            CK(ctx, cudaStreamWaitEvent(ctx->compute, s.ready, 0));
+            rc = accumulate_texture(ctx, s, take, sign);
+            if (rc) return rc;
+            CK(ctx, cudaEventRecord(s.consumed, ctx->compute));
+        }
+        if (refused) return refused;
     }
     return CPT_OK;
 }
@@ -693,7 +730,8 @@ int apply(composite_ctx *ctx, const void *members, int32_t n, int64_t stride, in
     if (kind == kDevice) {
         const bool aligned = (reinterpret_cast<uintptr_t>(members) % 16 == 0) && (pitch % 16 == 0) && (stride % 16 == 0);
         if (ctx->cfg.read_path == CPT_READ_TEXTURE) {
-            const bool direct = (ctx->width % ctx->vec_px == 0) && stride == (int64_t)pitch * ctx->height;
+            const bool direct = ctx->packed_array ||
+                                ((ctx->width % ctx->vec_px == 0) && stride == (int64_t)pitch * ctx->height);
             rc = direct ? run_texture_from_device(ctx, src, n, stride, pitch, sign)
                         : run_staged(ctx, src, n, stride, pitch, sign);
         } else if (aligned || ctx->cfg.read_path == CPT_READ_LINEAR) {

@@ -51,6 +51,13 @@ cudaError_t launch_count_texture(cudaTextureObject_t tex, int n_layers, const Pl
                                  int *flags, const DeviceCaps &caps, cudaStream_t s);
 cudaError_t launch_depth_texture(cudaTextureObject_t tex, int n_layers, const Plane &p, int sign,
                                  int *flags, const DeviceCaps &caps, cudaStream_t s);
+// The same over a mask array that holds one bit per pixel, 64 pixels to a
+// texel of two 32-bit words, and the conversion into it: member i of the batch
+// (any alignment) into layer i.
+int packed_texels(int width);
+cudaError_t launch_count_packed_texture(cudaTextureObject_t tex, int n_layers, const Plane &p, int sign, int *flags,
+                                        const DeviceCaps &caps, cudaStream_t s);
+cudaError_t launch_pack_to_array(const RasterBatch &b, int width, int height, cudaSurfaceObject_t surf, cudaStream_t s);
 // dst + i * stride <- src + ids[i] * stride, raster_bytes (a multiple of 16)
 // each, i < n; src may be host-mapped pinned memory.  16-byte aligned.
 cudaError_t launch_gather_rasters(void *dst, const void *src, const int32_t *ids, int n, int64_t stride,
