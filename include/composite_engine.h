@@ -7,7 +7,7 @@
  * The engine holds composite planes in device memory (uint32 or uint16 counts, one per
  * plane) and applies "ops" to them: add or remove a set of device-resident
  * uint8 masks to one plane.  All ops of one submit call run in ONE persistent
- * kernel launch whose warps pull work items (op, member slab, chunk of
+ * kernel launch whose CTAs pull work items (op, member slab, chunk of
  * 16-pixel groups) from a device counter, so small and large composites share
  * the GPU without one launch per composite; one render call likewise renders
  * many planes in one launch.  A submit + render sequence can be captured in a
@@ -47,15 +47,16 @@ typedef struct composite_engine composite_engine;
 
 /* How the accumulate launch hands work items to warps. */
 enum {
-    CPT_SCHEDULE_PERSISTENT = 0,  /* num_SMs x ctas_per_sm CTAs; warps claim items from a counter */
-    CPT_SCHEDULE_GRID = 1         /* one CTA per 8 items; the hardware schedules the CTAs        */
+    CPT_SCHEDULE_PERSISTENT = 0,  /* num_SMs x ctas_per_sm CTAs claim items from a counter */
+    CPT_SCHEDULE_GRID = 1         /* one CTA per item; the hardware schedules the CTAs       */
 };
 
 typedef struct composite_engine_config {
     void *cuda_stream;        /* cudaStream_t for all engine work, NULL = the legacy
                                  default stream (ordered with the caller's work there) */
     int32_t slab_members;     /* most members of an op per work item, 1..255; 0 = 128  */
-    int32_t ctas_per_sm;      /* persistent CTAs of 256 threads per SM, 1..8; 0 = 5   */
+    int32_t ctas_per_sm;      /* persistent CTAs of 256 threads per SM, 1..8; 0 = 5;
+                                 more than four run as four, all that fit             */
     int64_t wait_timeout_ms;  /* bound on host waits; 0 = 10000                        */
     int32_t schedule;         /* CPT_SCHEDULE_*; default CPT_SCHEDULE_PERSISTENT       */
     void *upload_stream;      /* cudaStream_t for the engine's small host-to-device
@@ -63,12 +64,10 @@ typedef struct composite_engine_config {
                                  that streams its own rasters on a copy stream passes
                                  it here so the small uploads queue behind its uploads
                                  in order instead of competing for a copy engine      */
-    int32_t item_member_groups; /* work item size: a lane folds at most about this many
-                                 (member, 16-pixel group) pairs per item, so an item
-                                 covers up to 32 x (item_member_groups / slab) groups
-                                 of one slab (fewer when a submit would otherwise give
-                                 the launch's warps fewer than four items each);
-                                 16..8192, 0 = 512                                      */
+    int32_t item_member_groups; /* work item size: a thread folds at most about this
+                                 many (member, 16-pixel group) pairs per item (fewer
+                                 when a submit would otherwise give the launch's CTAs
+                                 fewer than eight items each); 16..8192, 0 = 512        */
     int32_t staging_buffers;  /* staging buffers for host ops, 2..8; 0 = 2           */
     int64_t staging_bytes;    /* bytes per staging buffer, >= 1 MiB (and >= the largest
                                  host raster); 0 = 256 MiB.  Allocated at the first
@@ -184,7 +183,7 @@ int composite_engine_replay(composite_engine *eng);
 
 /* Autotuner: times "clear the ops' planes + submit ops", `repeats` runs per
  * candidate, in three passes, each keeping the fastest: (1) slab_members in
- * {32, 64, 128, 255} x schedule {grid, persistent with ctas_per_sm 3, 4, 5};
+ * {32, 64, 128, 255} x schedule {grid, persistent with ctas_per_sm 3, 4};
  * (2) item_member_groups in {256, 512, 1024, 2048} (the work item's tile of
  * groups); (3) when some op reads pinned host members, staging_buffers in
  * {2, 3, 4} x staging_bytes in {64, 128, 256, 512} MiB.  The winner becomes

@@ -1,19 +1,19 @@
 // engine.cu -- the batched composite engine of include/composite_engine.h.
 //
 // A submit turns every op (add/remove a member set to one plane) into work
-// items (op, member slab, chunk of 16-pixel groups), numbered op after op,
+// items (op, member slab, steps of 16-pixel groups), numbered op after op,
 // slab after slab, chunk after chunk.  One persistent launch of
-// num_SMs x ctas_per_sm CTAs runs warps that each pull item numbers from a
-// device counter; the op owning an item is found by binary search over the
-// ops' first items.  Each lane folds its groups of one slab's members into
-// packed byte counters (member i of the op read at base + idx(i) * stride,
-// the slab's indices staged in the warp's shared memory) and adds the counts
-// into the op's plane (uint32, or uint16 for a 16-bit plane): with L2
-// atomics, or with plain read-modify-writes when the plane's ops are single
-// slabs folded one after another by the same items (split_ops).  The render launch deals warp-level (plane,
-// 512 pixels) items round robin to its warps.  Consecutive
-// items are neighbouring chunks of the same slab, so concurrently running
-// warps read neighbouring bytes of the same members.
+// num_SMs x ctas_per_sm CTAs claims item numbers from a device counter; the
+// op owning an item is found by binary search over the ops' first items.  A
+// CTA folds its groups of one slab's members into packed byte counters
+// (member i of the op read at base + idx(i) * stride, the slab's indices
+// staged in shared memory) and adds the counts into the op's plane (uint32,
+// or uint16 for a 16-bit plane): with L2 atomics, or with plain
+// read-modify-writes when the plane's ops are single slabs folded one after
+// another by the same items (split_ops).  The render launch deals warp-level
+// (plane, 512 pixels) items round robin to its warps.  Consecutive items are
+// neighbouring chunks of the same slab, so concurrently running CTAs read
+// neighbouring bytes of the same members.
 #include <algorithm>
 #include <chrono>
 #include <cstdarg>
@@ -39,6 +39,9 @@ constexpr int kMaxPlanes = 1 << 16;
 constexpr int kMaxSlab = 255;          // packed byte counters
 constexpr int kUploadRing = 64;        // descriptor uploads in flight before the host waits
 constexpr int kSplitMembers = 32;      // shortest slab that a launch short of items is cut into
+constexpr int kSlices = 4;             // slices of a CTA's threads on items of kSliceMembers members or more
+constexpr int kSliceMembers = 32;
+constexpr int kResidentCtas = 4;       // CTAs per SM that the accumulate kernels' registers allow
 
 struct OpDesc {
     const uint8_t *base;
@@ -56,7 +59,8 @@ struct OpDesc {
     int32_t slab;
     int32_t sign;
     int32_t plane_id;
-    int32_t groups_per_thread;   // groups per lane per item (short slabs take several)
+    int32_t steps;               // steps per item: each kThreads / slices groups (or words)
+    int32_t slices;              // shares of a slab's members that the CTA's threads fold at once: 1 or 4
     int32_t exclusive;           // this chain is the only one on its plane, one slab: plain read-modify-write
     int32_t bits;                // bit-packed masks: a group is a 32-pixel word
     int32_t words_per_row;       // bits: ceil(width / 32)
@@ -192,51 +196,104 @@ __device__ __forceinline__ void apply_group(CountT *dst, const uint32_t (&k)[4],
         cpt::atomic_count_group<CountT>(dst, wide, op.sign, flags + op.plane_id);
 }
 
-// One warp item: (op, member slab, chunk of 32 x groups_per_thread groups),
-// and after the op's own slab those of the ops chained to it (one slab each,
-// the same plane and chunk): each op in turn adds to or takes from the
-// counts, by this lane alone.  The slab's member indices are staged in the
-// warp's slice of shared memory.
-__device__ __forceinline__ void process_item(const OpDesc *head, uint32_t item, int lane, int32_t *index,
-                                             int *flags) {
+// The same for one word of the packed counters, four pixels.
+template <typename CountT>
+__device__ __forceinline__ void apply_word(CountT *dst, uint32_t k, const OpDesc &op, int *flags) {
+    if (op.exclusive)
+        cpt::apply_count_word<CountT>(dst, k, op.sign, flags + op.plane_id);
+    else
+        cpt::atomic_count_word<CountT>(dst, k, op.sign, flags + op.plane_id);
+}
+
+// What a CTA shares while it works on an item: the slab's member ids, the
+// slices' packed counters.
+struct ItemShared {
+    int32_t index[kMaxSlab + 1];
+    uint4 part[kSlices][kThreads / kSlices];
+};
+
+// Row and first pixel of group (or word) g of rows of `per_row`.
+__device__ __forceinline__ int row_of(int64_t g, int per_row) {
+    return g <= 0xFFFFFFFFll ? (int)((uint32_t)g / (uint32_t)per_row) : (int)(g / per_row);
+}
+
+// The ids of op's slab from member m0 on into shared memory.
+__device__ __forceinline__ void stage_index(const OpDesc &op, int m0, int cnt, int32_t *index) {
+    for (int i = threadIdx.x; i < cnt; i += kThreads) index[i] = op.index[m0 + i];
+    __syncthreads();
+}
+
+// One CTA item: (op, member slab, `steps` steps of groups), and after the
+// op's own slab those of the ops chained to it (one slab each, the same plane
+// and groups): each op in turn adds to or takes from the counts, by the same
+// CTA alone.  With four slices a step is 64 groups whose members the slices
+// share, their counters added up in shared memory four pixels to a thread;
+// with one a thread folds its own group.
+__device__ __forceinline__ void process_item(const OpDesc *head, uint32_t item, ItemShared &sh, int *flags) {
     const uint32_t local = item - (uint32_t)head->item_start;
     const int sl = (int)(local / (uint32_t)head->tiles);
     const int chunk = (int)(local - (uint32_t)sl * head->tiles);
     const int64_t groups = (int64_t)head->groups_per_row * head->height;
-    const int gpt = head->groups_per_thread;
+    const int slices = head->slices;
+    const int span = kThreads / slices;
+    const int lane_group = threadIdx.x % span, slice = threadIdx.x / span;
+    const int64_t first = (int64_t)chunk * head->steps * span;
+    const int64_t last = min(groups, first + (int64_t)head->steps * span);
     const int chain = head->chain;
     for (int link = 0; link < chain; ++link) {
         const OpDesc &op = head[link];
         const int m0 = sl * op.slab;
         const int cnt = min(op.n - m0, op.slab);
         const bool gather = op.index != nullptr;
-        if (gather) {
-            for (int i = lane; i < cnt; i += 32) index[i] = op.index[m0 + i];
-            __syncwarp();
-        }
-        for (int j = 0; j < gpt; ++j) {
-            const int64_t g = ((int64_t)chunk * gpt + j) * 32 + lane;
-            if (g >= groups) break;
-            const int y = (int)(g / op.groups_per_row);
-            const int x0 = (int)(g - (int64_t)y * op.groups_per_row) * 16;
-            const int valid = min(16, op.width - x0);
-            // rows are at least a whole number of groups apart, so only the last
-            // row's right edge can end before its group does
-            const int exact = valid < 16 && y == op.height - 1 ? valid : 0;
-            const uint8_t *row = op.base + (int64_t)y * op.pitch + x0;
+        if (gather) stage_index(op, m0, cnt, sh.index);
+        const int share = (cnt + slices - 1) / slices;
+        const int i0 = min(cnt, slice * share);
+        const int mine = min(cnt, i0 + share) - i0;
+        for (int64_t base = first; base < last; base += span) {
+            const int64_t g = base + lane_group;
             uint32_t k[4] = {0u, 0u, 0u, 0u};
-            if (gather)
-                fold_group<true>(row, op.stride, m0, index, cnt, exact, k);
-            else
-                fold_group<false>(row, op.stride, m0, index, cnt, exact, k);
-            cpt::keep_valid(k, valid);
-            const int64_t at = (int64_t)y * op.plane_pitch + x0;
-            if (op.u16)
-                apply_group<uint16_t>(reinterpret_cast<uint16_t *>(op.plane) + at, k, op, flags);
-            else
-                apply_group<uint32_t>(op.plane + at, k, op, flags);
+            int64_t at = 0;
+            if (g < last) {
+                const int y = row_of(g, op.groups_per_row);
+                const int x0 = (int)(g - (int64_t)y * op.groups_per_row) * 16;
+                const int valid = min(16, op.width - x0);
+                // rows are at least a whole number of groups apart, so only the last
+                // row's right edge can end before its group does
+                const int exact = valid < 16 && y == op.height - 1 ? valid : 0;
+                const uint8_t *row = op.base + (int64_t)y * op.pitch + x0;
+                if (gather)
+                    fold_group<true>(row, op.stride, 0, sh.index + i0, mine, exact, k);
+                else
+                    fold_group<false>(row, op.stride, m0 + i0, nullptr, mine, exact, k);
+                cpt::keep_valid(k, valid);
+                at = (int64_t)y * op.plane_pitch + x0;
+            }
+            if (slices == 1) {
+                if (g >= last) continue;
+                if (op.u16)
+                    apply_group<uint16_t>(reinterpret_cast<uint16_t *>(op.plane) + at, k, op, flags);
+                else
+                    apply_group<uint32_t>(op.plane + at, k, op, flags);
+                continue;
+            }
+            sh.part[slice][lane_group] = make_uint4(k[0], k[1], k[2], k[3]);
+            __syncthreads();
+            const int64_t wg = base + threadIdx.x / 4;   // this thread's word of the step's 64 groups
+            if (wg < last) {
+                uint32_t sum = 0;
+#pragma unroll
+                for (int s = 0; s < kSlices; ++s) sum += reinterpret_cast<const uint32_t *>(sh.part[s])[threadIdx.x];
+                const int y = row_of(wg, op.groups_per_row);
+                const int64_t to = (int64_t)y * op.plane_pitch + (wg - (int64_t)y * op.groups_per_row) * 16 +
+                                   (threadIdx.x % 4) * 4;
+                if (op.u16)
+                    apply_word<uint16_t>(reinterpret_cast<uint16_t *>(op.plane) + to, sum, op, flags);
+                else
+                    apply_word<uint32_t>(op.plane + to, sum, op, flags);
+            }
+            __syncthreads();
         }
-        if (gather) __syncwarp();
+        if (gather) __syncthreads();
     }
 }
 
@@ -250,32 +307,28 @@ __device__ __forceinline__ uint32_t load_word(const uint8_t *q, int exact) {
     return v;
 }
 
-// The same for bit-packed masks: a lane owns 32-pixel words and keeps their
+// The same for bit-packed masks: a thread owns 32-pixel words and keeps their
 // counts in carry-save accumulators (BitCounter), 16 members per step.  Bits
 // past the raster's right edge are counted along and dropped from the
 // bit-slices at the end.
-__device__ __forceinline__ void process_bits_item(const OpDesc *head, uint32_t item, int lane, int32_t *index,
-                                                  int *flags) {
+__device__ __forceinline__ void process_bits_item(const OpDesc *head, uint32_t item, ItemShared &sh, int *flags) {
     const uint32_t local = item - (uint32_t)head->item_start;
     const int sl = (int)(local / (uint32_t)head->tiles);
     const int chunk = (int)(local - (uint32_t)sl * head->tiles);
     const int64_t words = (int64_t)head->words_per_row * head->height;
-    const int gpt = head->groups_per_thread;
+    const int64_t first = (int64_t)chunk * head->steps * kThreads;
+    const int64_t last = min(words, first + (int64_t)head->steps * kThreads);
     const int chain = head->chain;
+    const int32_t *index = sh.index;
     for (int link = 0; link < chain; ++link) {
         const OpDesc &op = head[link];
         const int m0 = sl * op.slab;
         const int cnt = min(op.n - m0, op.slab);
         const bool gather = op.index != nullptr;
-        if (gather) {
-            for (int i = lane; i < cnt; i += 32) index[i] = op.index[m0 + i];
-            __syncwarp();
-        }
+        if (gather) stage_index(op, m0, cnt, sh.index);
         const int64_t stride = op.stride;
-        for (int j = 0; j < gpt; ++j) {
-            const int64_t g = ((int64_t)chunk * gpt + j) * 32 + lane;
-            if (g >= words) break;
-            const int y = (int)(g / op.words_per_row);
+        for (int64_t g = first + threadIdx.x; g < last; g += kThreads) {
+            const int y = row_of(g, op.words_per_row);
             const int gx = (int)(g - (int64_t)y * op.words_per_row);
             const int x0 = gx * 32;
             const int valid = min(32, op.width - x0);
@@ -317,53 +370,56 @@ __device__ __forceinline__ void process_bits_item(const OpDesc *head, uint32_t i
                 }
             }
         }
-        if (gather) __syncwarp();
+        if (gather) __syncthreads();
     }
 }
 
-__device__ __forceinline__ void run_item(const OpDesc *head, uint32_t item, int lane, int32_t *index, int *flags) {
-    if (head->bits)
-        process_bits_item(head, item, lane, index, flags);
+// The mask formats of a launch's ops.  Each has a kernel of its own: the bit
+// counters' registers would otherwise be taken from the byte path, which had
+// to spill.
+enum Formats { kBytesOnly = 0, kBitsOnly = 1, kBothFormats = 2 };
+
+template <int kFormats>
+__device__ __forceinline__ void run_item(const OpDesc *head, uint32_t item, ItemShared &sh, int *flags) {
+    if (kFormats == kBitsOnly || (kFormats == kBothFormats && head->bits))
+        process_bits_item(head, item, sh, flags);
     else
-        process_item(head, item, lane, index, flags);
+        process_item(head, item, sh, flags);
 }
 
-// Persistent schedule: warps claim items from the counter one ahead (lane 0
-// asks for the next while the warp works on the current one), so warps
-// never wait for one another and uneven items balance across the GPU.
-// Two register budgets: launched with four or five CTAs per SM, 48 registers
-// (a few spill; four such CTAs still leave a quarter of the register file to
-// a kernel on another stream); with three or fewer, 64 and no spills (three
-// such CTAs leave the same quarter).
-template <int kCtasPerSm>
-__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+// Persistent schedule: CTA b takes item b, then claims items from the counter
+// (zero at launch) one ahead: thread 0 asks for the next while the CTA works
+// on the current one, and uneven items balance across the GPU.
+// At most four CTAs per SM are resident, on 64 registers: five on 48 spilled
+// and were slower (64 uneven requests with clear and render: 421 against 400
+// us).  Two or three of them leave room for a kernel on another stream.
+template <int kFormats>
+__global__ void __launch_bounds__(kThreads, kResidentCtas)
 engine_accumulate_kernel(const OpDesc *ops, int n_ops, uint32_t n_items, uint32_t *counter, int *flags) {
-    __shared__ int32_t s_index[kThreads / 32][kMaxSlab + 1];
+    __shared__ ItemShared sh;
     __shared__ uint32_t s_starts[kSmemStarts];
+    __shared__ uint32_t s_item;
     load_starts(ops, n_ops, s_starts);
     __syncthreads();
-    const int lane = threadIdx.x & 31;
-    int32_t *index = s_index[threadIdx.x >> 5];
-    uint32_t next = 0;
-    if (lane == 0) next = atomicAdd(counter, 1u);
-    next = __shfl_sync(0xFFFFFFFFu, next, 0);
-    while (next < n_items) {
-        const uint32_t item = next;
-        if (lane == 0) next = atomicAdd(counter, 1u);
-        run_item(ops + find_op(ops, n_ops, s_starts, item), item, lane, index, flags);
-        next = __shfl_sync(0xFFFFFFFFu, next, 0);
+    uint32_t item = blockIdx.x;
+    while (item < n_items) {
+        uint32_t next = 0;
+        if (threadIdx.x == 0) next = gridDim.x + atomicAdd(counter, 1u);
+        run_item<kFormats>(ops + find_op(ops, n_ops, s_starts, item), item, sh, flags);
+        if (threadIdx.x == 0) s_item = next;
+        __syncthreads();
+        item = s_item;
+        __syncthreads();
     }
 }
 
-// Grid schedule: one launch of ceil(items / 8) CTAs, warp w of CTA b takes
-// item 8b + w; the hardware block scheduler balances the CTAs.
-__global__ void __launch_bounds__(kThreads)
-engine_accumulate_grid_kernel(const OpDesc *ops, int n_ops, uint32_t n_items, int *flags) {
-    __shared__ int32_t s_index[kThreads / 32][kMaxSlab + 1];
-    const int lane = threadIdx.x & 31;
-    const uint32_t item = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
-    if (item >= n_items) return;
-    run_item(ops + find_desc(ops, n_ops, item), item, lane, s_index[threadIdx.x >> 5], flags);
+// Grid schedule: a CTA per item; the hardware block scheduler balances them.
+template <int kFormats>
+__global__ void __launch_bounds__(kThreads, kResidentCtas)
+engine_accumulate_grid_kernel(const OpDesc *ops, int n_ops, int *flags) {
+    __shared__ ItemShared sh;
+    const uint32_t item = blockIdx.x;
+    run_item<kFormats>(ops + find_desc(ops, n_ops, item), item, sh, flags);
 }
 
 // Clear of many planes in one launch (counts to zero, the planes' underflow
@@ -377,7 +433,7 @@ engine_clear_kernel(const ClearDesc *ops, int n_ops, uint32_t n_items, int *flag
     __syncthreads();
     if (blockIdx.x == 0)
         for (int i = threadIdx.x; i < n_ops; i += blockDim.x)
-            if (ops[i].plane_id >= 0) flags[ops[i].plane_id] = 0;   // -1: a histogram, no flag
+            if (ops[i].plane_id >= 0) flags[ops[i].plane_id] = 0;   // -1: a histogram or a counter, no flag
     const int lane = threadIdx.x & 31;
     const uint32_t warps = gridDim.x * (kThreads / 32);
     const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
@@ -570,7 +626,6 @@ struct composite_engine {
     std::vector<PlaneRec> planes;
     int *d_flags = nullptr;
     int *h_flags = nullptr;
-    uint32_t *d_counter = nullptr;
     Upload up_ops[kUploadRing], up_render[kUploadRing];
     int up_i = 0, rup_i = 0;
     cudaEvent_t done_ev = nullptr;
@@ -652,6 +707,16 @@ Lut make_lut(const uint8_t *rgba) {
     return l;
 }
 
+// Bytes ahead of a submit's op descriptors: the item counter, zero.
+constexpr size_t kCounterBytes = 16;
+
+// Op descriptors as a submit uploads them.
+std::vector<unsigned char> op_blob(const std::vector<OpDesc> &descs) {
+    std::vector<unsigned char> blob(kCounterBytes + descs.size() * sizeof(OpDesc), 0);
+    if (!descs.empty()) memcpy(blob.data() + kCounterBytes, descs.data(), descs.size() * sizeof(OpDesc));
+    return blob;
+}
+
 // Copies `bytes` of descriptors into the next slot of the upload ring
 // and queues their upload, on the upload stream when the engine has one (so
 // that small uploads follow the caller's own uploads in order instead of
@@ -727,24 +792,33 @@ bool plane_ok(const composite_engine *e, int32_t p) {
 // at a time.  A plane's ops chain when each is one slab, all have one mask
 // format and they hold at most item_member_groups members together.
 //
-// Parallelism.  A launch runs num_SMs x ctas_per_sm x 8 warps.  Where its
-// planes' groups alone do not give every warp an item, chains and slabs of
-// more than kSplitMembers members are cut into slabs of down to that many --
-// but not chains that both add and remove: folded in order, a member added
-// and taken away in one submit never looks like an underflow.
-// A lane's work on an item is at most item_member_groups (member, group)
-// pairs, and less where the launch would otherwise have fewer than four
-// items per warp.  Measured on eight sessions' adds and removes of about 26
+// Slices.  From kSliceMembers members on, a slab's members are shared by four
+// slices of the CTA (see count_kernels.cu, where the split was measured).
+//
+// Parallelism.  A launch runs num_SMs x ctas_per_sm CTAs (at most four per
+// SM).  Where its planes'
+// groups alone do not give every CTA an item, chains and slabs of more than
+// kSplitMembers members are cut into slabs of down to that many -- but not
+// chains that both add and remove: folded in order, a member added and taken
+// away in one submit never looks like an underflow.
+// A thread's work on an item is at most item_member_groups (member, group)
+// pairs, and less where the launch would otherwise have fewer than eight
+// items per CTA.  Measured on eight sessions' adds and removes of about 26
 // overflow rasters of 1024^2: 15 CTAs and 1.66 ms in items of 512 pairs; a
-// whole served pass 2.88 ms with such items and atomics, 0.58 ms with these.
+// whole served pass 2.88 ms with such items and atomics, 0.47 ms now.  Items
+// of single warps (no slices) took 420 us for the 64 uneven requests' 2.0 GB
+// of masks, items of CTAs take 350 (5.8 TB/s).
 int64_t split_ops(const composite_engine *e, std::vector<OpDesc> *descs) {
-    const int64_t warps = (int64_t)e->caps.num_sms * e->cfg.ctas_per_sm * (kThreads / 32);
+    const int64_t ctas = (int64_t)e->caps.num_sms * std::min(e->cfg.ctas_per_sm, kResidentCtas);
     const int cfg_slab = e->cfg.slab_members;
-    auto warp_tiles = [](const OpDesc &d) {   // items of one group (or word) per lane
-        return ((int64_t)(d.bits ? d.words_per_row : d.groups_per_row) * d.height + 31) / 32;
+    auto slices_of = [](const OpDesc &d, int members) { return !d.bits && members >= kSliceMembers ? kSlices : 1; };
+    auto steps_of = [](const OpDesc &d, int slices) {   // steps over the whole plane
+        const int64_t span = kThreads / slices;
+        return ((int64_t)(d.bits ? d.words_per_row : d.groups_per_row) * d.height + span - 1) / span;
     };
     struct PlaneOps {
         int64_t members = 0;
+        int most = 0;           // members of its longest op
         int ops = 0;
         int32_t bits = -1;      // the ops' mask format, -2 when they differ
         bool single = true;     // every op is one slab
@@ -752,22 +826,23 @@ int64_t split_ops(const composite_engine *e, std::vector<OpDesc> *descs) {
         bool chained = false;
     };
     std::vector<PlaneOps> planes(e->planes.size());
-    int64_t tiles_once = 0;      // warp tiles of the planes' first ops
-    int64_t lane_work = 0;       // (member, group) pairs per lane over all warp tiles
+    int64_t steps_once = 0;      // steps of the planes' first ops
+    int64_t thread_work = 0;     // (member, group) pairs per thread over all steps
     for (const OpDesc &d : *descs) {
         PlaneOps &p = planes[d.plane_id];
         if (p.ops++ == 0) {
             p.bits = d.bits;
-            tiles_once += warp_tiles(d);
+            steps_once += steps_of(d, slices_of(d, d.n));
         } else if (p.bits != d.bits) {
             p.bits = -2;
         }
         p.members += d.n;
         p.single = p.single && d.n <= cfg_slab;
         (d.sign > 0 ? p.adds : p.removes) = true;
-        lane_work += warp_tiles(d) * d.n;
+        p.most = std::max(p.most, d.n);
+        thread_work += steps_of(d, 1) * d.n;
     }
-    const bool fills = tiles_once >= warps;
+    const bool fills = steps_once >= ctas;
     for (PlaneOps &p : planes)
         p.chained = p.ops > 0 && p.single && p.bits >= 0 && p.members <= std::max(cfg_slab, e->cfg.item_member_groups) &&
                     (fills || p.members <= kSplitMembers || (p.adds && p.removes));
@@ -790,7 +865,7 @@ int64_t split_ops(const composite_engine *e, std::vector<OpDesc> *descs) {
         }
         descs->swap(order);
     }
-    const int64_t target = std::min<int64_t>(e->cfg.item_member_groups, std::max<int64_t>(16, lane_work / (4 * warps)));
+    const int64_t target = std::min<int64_t>(e->cfg.item_member_groups, std::max<int64_t>(8, thread_work / (8 * ctas)));
     int64_t items = 0;
     for (size_t i = 0; i < descs->size();) {
         OpDesc &head = (*descs)[i];
@@ -798,13 +873,14 @@ int64_t split_ops(const composite_engine *e, std::vector<OpDesc> *descs) {
         const int chain = p.chained ? p.ops : 1;
         int slab = cfg_slab;
         if (!p.chained && !fills && head.n > kSplitMembers) {
-            const int64_t parts = (warps + tiles_once - 1) / tiles_once;
+            const int64_t parts = (ctas + steps_once - 1) / steps_once;
             slab = (int)std::min<int64_t>(slab, std::max<int64_t>(kSplitMembers, (head.n + parts - 1) / parts));
         }
-        const int64_t per_lane = p.chained ? p.members : std::min(head.n, slab);
-        const int64_t tiles1 = warp_tiles(head);
-        head.groups_per_thread = (int32_t)std::max<int64_t>(1, target / per_lane);
-        head.tiles = (int32_t)((tiles1 + head.groups_per_thread - 1) / head.groups_per_thread);
+        head.slices = slices_of(head, p.chained ? p.most : std::min(head.n, slab));
+        const int64_t per_thread = (p.chained ? p.members : std::min(head.n, slab)) / head.slices;
+        const int64_t steps = steps_of(head, head.slices);
+        head.steps = (int32_t)std::max<int64_t>(1, std::min<int64_t>(steps, target / std::max<int64_t>(1, per_thread)));
+        head.tiles = (int32_t)((steps + head.steps - 1) / head.steps);
         head.slab = slab;
         head.chain = chain;
         head.exclusive = p.chained || (p.ops == 1 && head.n <= slab) ? 1 : 0;
@@ -933,29 +1009,40 @@ int plan_render(composite_engine *e, const composite_render_op *ops, int32_t n_o
 }
 
 unsigned persistent_grid(const composite_engine *e, int64_t items) {
-    const int64_t cap = (int64_t)e->caps.num_sms * e->cfg.ctas_per_sm;
+    const int64_t cap = (int64_t)e->caps.num_sms * std::min(e->cfg.ctas_per_sm, kResidentCtas);
     return (unsigned)std::max<int64_t>(1, std::min(cap, items));
 }
 
-int launch_accumulate(composite_engine *e, const void *d_ops, int n_ops, int64_t n_items, uint32_t *counter) {
-    if (e->cfg.schedule == CPT_SCHEDULE_GRID) {
-        const int64_t ctas = (n_items + kThreads / 32 - 1) / (kThreads / 32);
-        engine_accumulate_grid_kernel<<<(unsigned)ctas, kThreads, 0, e->stream>>>(
-            static_cast<const OpDesc *>(d_ops), n_ops, (uint32_t)n_items, e->d_flags);
-    } else {
-        ECK(e, cudaMemsetAsync(counter, 0, sizeof(uint32_t), e->stream));
-        const int64_t warps_needed = (n_items + kThreads / 32 - 1) / (kThreads / 32);
-        const unsigned grid = (unsigned)std::min<int64_t>(persistent_grid(e, n_items), warps_needed);
-        const OpDesc *ops = static_cast<const OpDesc *>(d_ops);
-        if (e->cfg.ctas_per_sm >= 4)
-            engine_accumulate_kernel<5><<<grid, kThreads, 0, e->stream>>>(ops, n_ops, (uint32_t)n_items, counter,
-                                                                          e->d_flags);
-        else
-            engine_accumulate_kernel<4><<<grid, kThreads, 0, e->stream>>>(ops, n_ops, (uint32_t)n_items, counter,
-                                                                          e->d_flags);
-    }
+template <int kFormats>
+void launch_accumulate_t(composite_engine *e, const OpDesc *ops, int n_ops, int64_t n_items, uint32_t *counter) {
+    const unsigned grid = persistent_grid(e, n_items);
+    const uint32_t items = (uint32_t)n_items;
+    if (e->cfg.schedule == CPT_SCHEDULE_GRID)
+        engine_accumulate_grid_kernel<kFormats><<<items, kThreads, 0, e->stream>>>(ops, n_ops, e->d_flags);
+    else
+        engine_accumulate_kernel<kFormats><<<grid, kThreads, 0, e->stream>>>(ops, n_ops, items, counter, e->d_flags);
+}
+
+// counter: a zeroed device word (persistent schedule).
+int launch_accumulate(composite_engine *e, const void *d_ops, const std::vector<OpDesc> &descs, int64_t n_items,
+                      uint32_t *counter) {
+    bool bytes = false, bits = false;
+    for (const OpDesc &d : descs) (d.bits ? bits : bytes) = true;
+    const OpDesc *ops = static_cast<const OpDesc *>(d_ops);
+    const int n_ops = (int)descs.size();
+    if (!bits)
+        launch_accumulate_t<kBytesOnly>(e, ops, n_ops, n_items, counter);
+    else if (!bytes)
+        launch_accumulate_t<kBitsOnly>(e, ops, n_ops, n_items, counter);
+    else
+        launch_accumulate_t<kBothFormats>(e, ops, n_ops, n_items, counter);
     ECK(e, cudaGetLastError());
     return CPT_OK;
+}
+
+int launch_uploaded(composite_engine *e, const std::vector<OpDesc> &descs, int64_t items, void *blob) {
+    return launch_accumulate(e, static_cast<unsigned char *>(blob) + kCounterBytes, descs, items,
+                             static_cast<uint32_t *>(blob));
 }
 
 // True when some render op asks for a class histogram.
@@ -1119,11 +1206,12 @@ int launch_ops(composite_engine *e, const composite_op *ops, int32_t n_ops, bool
     int rc = plan_ops(e, ops, n_ops, &descs, &items, &n_after, false, false);
     if (rc || items == 0) return rc;
     Upload *u = nullptr;
-    rc = upload(e, e->up_ops, &e->up_i, descs.data(), descs.size() * sizeof(OpDesc), &u, desc_stream);
+    const std::vector<unsigned char> blob = op_blob(descs);
+    rc = upload(e, e->up_ops, &e->up_i, blob.data(), blob.size(), &u, desc_stream);
     if (rc) return rc;
     if (cpt::fault_injected("engine_submit")) return efail(e, CPT_ECUDA, "submit refused before its launch (injected)");
     *launched = true;   // from here on the launch may have begun
-    rc = launch_accumulate(e, u->d, (int)descs.size(), items, e->d_counter);
+    rc = launch_uploaded(e, descs, items, u->d);
     if (rc) return rc;
     ECK(e, cudaEventRecord(u->consumed, e->stream));
     return CPT_OK;
@@ -1238,12 +1326,13 @@ int submit_internal(composite_engine *e, const composite_op *ops, int32_t n_ops)
     if (host_ops.empty()) {
         if (items > 0) {
             Upload *u = nullptr;
-            rc = upload(e, e->up_ops, &e->up_i, descs.data(), descs.size() * sizeof(OpDesc), &u);
+            const std::vector<unsigned char> blob = op_blob(descs);
+            rc = upload(e, e->up_ops, &e->up_i, blob.data(), blob.size(), &u);
             if (rc) return rc;   // nothing launched: every plane is as before
             if (cpt::fault_injected("engine_submit"))
                 return efail(e, CPT_ECUDA, "submit refused before its launch (injected)");
             launched = true;
-            rc = launch_accumulate(e, u->d, (int)descs.size(), items, e->d_counter);
+            rc = launch_uploaded(e, descs, items, u->d);
             if (!rc) {
                 for (const auto &pn : n_after) e->planes[pn.first].n = pn.second;
                 ECK(e, cudaEventRecord(u->consumed, e->stream));
@@ -1293,7 +1382,6 @@ void destroy_engine(composite_engine *e) {
         }
     if (e->d_flags) cudaFree(e->d_flags);
     if (e->h_flags) cudaFreeHost(e->h_flags);
-    if (e->d_counter) cudaFree(e->d_counter);
     if (e->done_ev) cudaEventDestroy(e->done_ev);
     if (e->capture_stream) cudaStreamDestroy(e->capture_stream);
     free_stage(e);
@@ -1355,7 +1443,6 @@ int composite_engine_begin(composite_engine **out, const composite_engine_config
         ECK(e, cudaMalloc(&e->d_flags, kMaxPlanes * sizeof(int)));
         ECK(e, cudaMemsetAsync(e->d_flags, 0, kMaxPlanes * sizeof(int), e->stream));
         ECK(e, cudaHostAlloc(&e->h_flags, kMaxPlanes * sizeof(int), cudaHostAllocDefault));
-        ECK(e, cudaMalloc(&e->d_counter, sizeof(uint32_t)));
         ECK(e, cudaEventCreateWithFlags(&e->done_ev, cudaEventDisableTiming));
         for (Upload *ring : {e->up_ops, e->up_render})
             for (int i = 0; i < kUploadRing; ++i) {
@@ -1534,7 +1621,15 @@ int composite_engine_capture(composite_engine *e, const composite_op *ops, int32
     rc = drain(e);
     if (rc) return rc;
     destroy_graph(e);
-    ECK(e, cudaMalloc(&e->graph_counters, 2 * sizeof(uint32_t)));
+    ECK(e, cudaMalloc(&e->graph_counters, kCounterBytes));
+    if (items > 0) {   // the item counter too
+        ClearDesc d{};
+        d.data = reinterpret_cast<uint4 *>(e->graph_counters);
+        d.words = kCounterBytes / 16;
+        d.item_start = citems++;
+        d.plane_id = -1;
+        cdescs.push_back(d);
+    }
     if (!cdescs.empty()) {
         ECK(e, cudaMalloc(&e->graph_clears, cdescs.size() * sizeof(ClearDesc)));
         ECK(e, cudaMemcpy(e->graph_clears, cdescs.data(), cdescs.size() * sizeof(ClearDesc), cudaMemcpyHostToDevice));
@@ -1565,7 +1660,7 @@ int composite_engine_capture(composite_engine *e, const composite_op *ops, int32
             if (r) return r;
         }
         if (items > 0) {
-            int r = launch_accumulate(e, e->graph_ops, (int)descs.size(), items, e->graph_counters);
+            int r = launch_accumulate(e, e->graph_ops, descs, items, e->graph_counters);
             if (r) return r;
         }
         if (ritems > 0) {
@@ -1664,7 +1759,7 @@ int composite_engine_tune(composite_engine *e, const composite_op *ops, int32_t 
     };
     // pass 1: slab depth x schedule (ctas_per_sm 0 stands for the grid schedule)
     static const int slabs[] = {32, 64, 128, 255};
-    static const int ctas[] = {0, 3, 4, 5};
+    static const int ctas[] = {0, 3, 4};
     const int ctas_before = e->cfg.ctas_per_sm;
     for (int sl : slabs)
         for (int c : ctas) {

@@ -62,6 +62,31 @@ def test_adds_and_removes_of_many_planes(adds, removes, fmt, count_bits):
             np.testing.assert_array_equal(got, want)
 
 
+@pytest.mark.parametrize("schedule", ["persistent", "grid"])
+@pytest.mark.parametrize("fmt", ["bytes", "bits"])
+def test_few_long_ops_are_split_and_replayed(fmt, schedule):
+    # too few groups for every CTA: slabs of down to 32 members by atomics; slices of 4 at 32 members and more
+    sizes = [(40, 9, 31), (96, 33, 32), (513, 5, 255), (300, 70, 700)]
+    with binding.Engine(schedule=schedule) as eng:
+        ops, rops, checks = [], [], []
+        for i, (w, h, n) in enumerate(sizes):
+            m = synth.random_masks(70 + i, n, h, w)
+            plane = eng.add_plane(w, h)
+            counts = torch.empty((h, w), dtype=torch.int32, device="cuda")
+            ops.append(eng.op(plane, tight(synth.pack_masks(m) if fmt == "bits" else m), mask_format=fmt))
+            rops.append(eng.render_op(plane, counts))
+            checks.append((counts, oracle.count(m)))
+        keep = list(eng._keep)
+        eng.capture(ops, rops, keep=keep)
+        for _ in range(3):   # the item counter starts every replay from zero
+            for counts, _c in checks:
+                counts.fill_(-1)
+            eng.replay()
+            eng.sync()
+            for counts, c in checks:
+                np.testing.assert_array_equal(counts.cpu().numpy(), c)
+
+
 def test_mixed_formats_and_underflow_on_one_plane():
     w, h = 200, 50
     a, b = synth.random_masks(1, 40, h, w), synth.random_masks(2, 12, h, w)
