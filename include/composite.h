@@ -287,7 +287,7 @@ const char *composite_last_error(const composite_ctx *ctx);
  * composite_last_error(NULL). */
 int composite_selftest_bounded_wait(int64_t timeout_us, int32_t *gave_up_out, int64_t *waited_us_out);
 
-/* Largest composite plane of composite_oneshot_static, in padded pixels:
+/* Largest raster of composite_oneshot_static, in padded pixels:
  * roundup(width, 16) * height must not exceed it (2048 x 2048). */
 #define CPT_ONESHOT_MAX_PIXELS 4194304
 
@@ -309,14 +309,9 @@ int composite_selftest_bounded_wait(int64_t timeout_us, int32_t *gave_up_out, in
  * default.
  * The work is queued on cuda_stream (a cudaStream_t, NULL = legacy default
  * stream) and the call returns without waiting.
- * Scratch: a file-scope __device__ array of CPT_ONESHOT_MAX_PIXELS uint32
- * counts (16 MiB, plus 16 bytes of flags) that every GPU loading the library
- * holds until the process exits.  The first call on a device looks up its
- * address (cudaGetSymbolAddress) and should come before any stream capture.
- * Every call on a device shares that array and clears the part it uses, so
- * calls whose work overlaps on the GPU (different streams, or host threads)
- * race and must be serialised by the caller.
- * Errors: CPT_EINVAL (empty raster, raster larger than the scratch,
+ * One kernel, no scratch: nothing is shared between calls, which may overlap
+ * on the GPU (different streams, or host threads) and may be captured.
+ * Errors: CPT_EINVAL (empty raster, raster larger than the limit,
  * unaligned members or outputs, members or outputs not in the current
  * device's memory, bad strides), CPT_ECUDA; the message is in
  * composite_last_error(NULL). */

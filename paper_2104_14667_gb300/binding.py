@@ -319,7 +319,7 @@ def _check_static_outputs(members, h, w, counts_out, bucket_out, rgba_out):
 def composite_oneshot_static(members, counts_out=None, bucket_out=None, rgba_out=None, lut=None,
                              stream=None) -> None:
     """One-shot composite of device-resident masks with no allocation in the
-    library (scratch in a fixed device array); queued on ``stream``."""
+    library (one kernel, no scratch); queued on ``stream``."""
     lib = load()
     ptr, n, h, w, stride, pitch, dtype, _ = _raster_view(members)
     if dtype is not np.uint8:

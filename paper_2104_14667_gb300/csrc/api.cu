@@ -505,8 +505,19 @@ Slot &next_slot(composite_ctx *ctx) {
     return ctx->slots[ctx->next_slot++ % ctx->slots.size()];
 }
 
+// Work on the copy stream starts after the caller's earlier work on the
+// compute stream (which may have produced the rasters).  Rasters read in place
+// need no copy stream, and no such hand-over.
+int open_copy(composite_ctx *ctx) {
+    CK(ctx, cudaEventRecord(ctx->caller_ready, ctx->compute));
+    CK(ctx, cudaStreamWaitEvent(ctx->copy, ctx->caller_ready, 0));
+    return CPT_OK;
+}
+
 // Pinned-host or device rasters: upload chunk by chunk through the slots.
 int run_staged(composite_ctx *ctx, const uint8_t *src, int n, int64_t stride, int64_t pitch, int sign) {
+    const int orc = open_copy(ctx);
+    if (orc) return orc;
     const int C = ctx->call_chunk;
     for (int m0 = 0; m0 < n; m0 += C) {
         const cpt::TraceRange chunk_range("composite chunk");
@@ -537,6 +548,8 @@ int run_staged(composite_ctx *ctx, const uint8_t *src, int n, int64_t stride, in
 // one stream for the other); the first of the chunks gets a trace record of
 // the conversion's interval, the others empty ones at its end.
 int run_texture_from_device(composite_ctx *ctx, const uint8_t *src, int n, int64_t stride, int64_t pitch, int sign) {
+    const int orc = open_copy(ctx);
+    if (orc) return orc;
     const int C = ctx->call_chunk;
     int per_array = ctx->packed_array ? std::max(C, ctx->array_layers / C * C) : C;
     // in equal parts, whole chunks each: a short last one would be a conversion and a fold for little
@@ -573,6 +586,8 @@ int run_texture_from_device(composite_ctx *ctx, const uint8_t *src, int n, int64
 constexpr int64_t kIngestPiece = 4 << 20;   // bytes per ring-copy piece
 
 int run_ring(composite_ctx *ctx, const uint8_t *src, int n, int64_t stride, int64_t pitch, int sign) {
+    const int orc = open_copy(ctx);
+    if (orc) return orc;
     const int k = (int)ctx->slots.size();
     if (ctx->ring_chunk == 0) {
         int64_t chunk = ctx->slot_members;
@@ -722,10 +737,6 @@ int apply(composite_ctx *ctx, const void *members, int32_t n, int64_t stride, in
         return fail(ctx, CPT_EINVAL, "members are device memory of another GPU (the context runs on device %d)", ctx->device);
     ctx->call_chunks = 0;
     ctx->call_chunk = chunk_for_call(ctx, n);
-    // uploads on the copy stream start after the caller's earlier work on the
-    // compute stream (which may have produced the rasters)
-    CK(ctx, cudaEventRecord(ctx->caller_ready, ctx->compute));
-    CK(ctx, cudaStreamWaitEvent(ctx->copy, ctx->caller_ready, 0));
     int rc;
     if (kind == kDevice) {
         const bool aligned = (reinterpret_cast<uintptr_t>(members) % 16 == 0) && (pitch % 16 == 0) && (stride % 16 == 0);
@@ -966,8 +977,7 @@ int composite_clear(composite_ctx *ctx) try {
                          (ctx->cfg.mode == CPT_MODE_COUNT ? ctx->cfg.count_bits / 8 : 4);
     ctx->trace.clear();
     ctx->trace_used = 0;
-    CK(ctx, cudaMemsetAsync(ctx->plane.data, 0, bytes, ctx->compute));
-    CK(ctx, cudaMemsetAsync(ctx->flags, 0, cpt::kFlagCount * sizeof(int), ctx->compute));
+    CK(ctx, cpt::launch_clear_plane(ctx->plane.data, (int64_t)bytes, ctx->flags, ctx->caps, ctx->compute));
     ctx->n_members = 0;
     ctx->poisoned = false;
     memset(ctx->h_flags, 0, cpt::kFlagCount * sizeof(int));

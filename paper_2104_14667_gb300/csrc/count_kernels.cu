@@ -270,7 +270,22 @@ cudaError_t launch_depth_t(const RasterBatch &b, const Plane &p, int sign, const
     return cudaGetLastError();
 }
 
+// Counts (or sums) and device flags to zero, in one launch.
+__global__ void __launch_bounds__(kThreads)
+clear_plane_kernel(uint4 *data, int64_t words, int *flags) {
+    if (blockIdx.x == 0 && threadIdx.x < kFlagCount) flags[threadIdx.x] = 0;
+    for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < words; i += (int64_t)gridDim.x * kThreads)
+        data[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 }  // namespace
+
+cudaError_t launch_clear_plane(void *data, int64_t bytes, int *flags, const DeviceCaps &caps, cudaStream_t s) {
+    const int64_t words = bytes / 16;   // plane rows are whole 16-byte vectors
+    const int64_t blocks = std::min<int64_t>((words + 4 * kThreads - 1) / (4 * kThreads), 8ll * caps.num_sms);
+    clear_plane_kernel<<<(unsigned)std::max<int64_t>(1, blocks), kThreads, 0, s>>>(static_cast<uint4 *>(data), words, flags);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_count_linear(const RasterBatch &b, const Plane &p, int sign, int *flags,
                                 const DeviceCaps &caps, cudaStream_t s) {

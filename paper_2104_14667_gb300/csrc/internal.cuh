@@ -35,6 +35,9 @@ struct DeviceCaps {
     int num_sms;
 };
 
+// Clears a plane and the device flags (one launch: a memset each took two).
+cudaError_t launch_clear_plane(void *data, int64_t bytes, int *flags, const DeviceCaps &caps, cudaStream_t s);
+
 // Linear read path: 16-byte loads straight from the batch (device memory).
 cudaError_t launch_count_linear(const RasterBatch &b, const Plane &p, int sign, int *flags,
                                 const DeviceCaps &caps, cudaStream_t s);
