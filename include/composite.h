@@ -147,7 +147,8 @@ typedef struct composite_config {
                                    (the paper's pipeline); default 0                      */
     int32_t tma_box_bytes;      /* CPT_READ_TMA box width in bytes: 64, 128 or 256 (a box is
                                    2 KiB per member: width x 2048/width rows, x 16 members);
-                                   0 = 256                                                */
+                                   0 = 2 KiB of consecutive rows where the rasters have no
+                                   row padding, else 256                                  */
     int32_t mask_format;        /* CPT_MASK_*; CPT_MASK_BITS needs CPT_MODE_COUNT and
                                    CPT_READ_LINEAR; default CPT_MASK_BYTES                */
     int32_t layout_converter;   /* CPT_READ_TEXTURE: how rasters reach the cudaArray;

@@ -397,6 +397,11 @@ int setup(composite_ctx *ctx) {
     return CPT_OK;
 }
 
+// Whether the TMA path reads a batch as runs (tma_box_bytes 0 and unpadded rows).
+bool tma_runs(const composite_ctx *ctx, const RasterBatch &b) {
+    return ctx->cfg.tma_box_bytes == 0 && cpt::tma_run_compatible(b, ctx->width, ctx->height, ctx->elem);
+}
+
 // The accumulation kernel over one batch already in device memory (a staging
 // slot, or the caller's own rasters when they can be read in place), or in
 // pinned host memory read through its device mapping (host_mapped: only the
@@ -409,8 +414,10 @@ int accumulate(composite_ctx *ctx, const RasterBatch &b, int sign, bool host_map
     cudaError_t e;
     if (ctx->cfg.read_path == CPT_READ_TMA) {
         CUtensorMap map;
-        const int box = ctx->cfg.tma_box_bytes;
-        const int r = cpt::encode_tma_map(&map, b, ctx->width, ctx->height, ctx->elem, box);
+        const bool runs = tma_runs(ctx, b);
+        const int box = runs ? cpt::kTmaRuns : ctx->cfg.tma_box_bytes ? ctx->cfg.tma_box_bytes : kDefaultTmaBoxBytes;
+        const int r = runs ? cpt::encode_tma_run_map(&map, b, ctx->width, ctx->height, ctx->elem)
+                           : cpt::encode_tma_map(&map, b, ctx->width, ctx->height, ctx->elem, box);
         if (r != 0) return fail(ctx, CPT_ECUDA, "cuTensorMapEncodeTiled failed (CUresult %d)", r);
         e = count ? cpt::launch_count_tma(map, b, ctx->plane, sign, ctx->flags, tns, box, ctx->caps, ctx->compute)
                   : cpt::launch_depth_tma(map, b, ctx->plane, sign, ctx->flags, tns, box, ctx->caps, ctx->compute);
@@ -482,14 +489,19 @@ int consume_slot(composite_ctx *ctx, Slot &s, int c, int sign) {
     return accumulate(ctx, b, sign);
 }
 
-// Uploads c rasters (any memory kind) into a staging buffer laid out with
-// row pitch pitch_px * elem and raster stride member_bytes.
+// Uploads c rasters (pinned host or device memory) into a staging buffer laid
+// out with row pitch stage_pitch and raster stride member_bytes.  Device
+// rasters go by a kernel: as pitched copies, 154-pixel depth rows moved at
+// 1 TB/s.
 int upload(composite_ctx *ctx, uint8_t *dst, const uint8_t *src, int c, int64_t stride,
-           int64_t pitch) {
+           int64_t pitch, bool device) {
     const int64_t row = ctx->row_bytes;
     const int64_t dpitch = ctx->stage_pitch;
     const int64_t h = ctx->height;
-    if (pitch == row && row == dpitch && stride == pitch * h) {
+    if (device) {
+        CK(ctx, cpt::launch_repitch(dst, dpitch, ctx->member_bytes, RasterBatch{src, stride, pitch, c}, row, ctx->height,
+                                    ctx->copy));
+    } else if (pitch == row && row == dpitch && stride == pitch * h) {
         CK(ctx, cudaMemcpyAsync(dst, src, (size_t)c * ctx->member_bytes, cudaMemcpyDefault, ctx->copy));
     } else if (stride == pitch * h) {
         CK(ctx, cudaMemcpy2DAsync(dst, dpitch, src, pitch, row, (size_t)c * h, cudaMemcpyDefault, ctx->copy));
@@ -515,7 +527,8 @@ int open_copy(composite_ctx *ctx) {
 }
 
 // Pinned-host or device rasters: upload chunk by chunk through the slots.
-int run_staged(composite_ctx *ctx, const uint8_t *src, int n, int64_t stride, int64_t pitch, int sign) {
+int run_staged(composite_ctx *ctx, const uint8_t *src, int n, int64_t stride, int64_t pitch, int sign,
+               bool device = false) {
     const int orc = open_copy(ctx);
     if (orc) return orc;
     const int C = ctx->call_chunk;
@@ -528,7 +541,7 @@ int run_staged(composite_ctx *ctx, const uint8_t *src, int n, int64_t stride, in
         CK(ctx, cudaStreamWaitEvent(ctx->copy, s.consumed, 0));
         rc = trace_open(ctx, kTraceUpload, ctx->copy);
         if (rc) return rc;
-        rc = upload(ctx, s.stage, src + (int64_t)m0 * stride, c, stride, pitch);
+        rc = upload(ctx, s.stage, src + (int64_t)m0 * stride, c, stride, pitch, device);
         if (rc) return rc;
         rc = trace_close(ctx, ctx->copy);
         if (rc) return rc;
@@ -744,15 +757,16 @@ int apply(composite_ctx *ctx, const void *members, int32_t n, int64_t stride, in
             const bool direct = ctx->packed_array ||
                                 ((ctx->width % ctx->vec_px == 0) && stride == (int64_t)pitch * ctx->height);
             rc = direct ? run_texture_from_device(ctx, src, n, stride, pitch, sign)
-                        : run_staged(ctx, src, n, stride, pitch, sign);
-        } else if (aligned || ctx->cfg.read_path == CPT_READ_LINEAR) {
-            // read in place: the linear kernels take any alignment, the tensor
-            // map 16 bytes
+                        : run_staged(ctx, src, n, stride, pitch, sign, true);
+        } else if (aligned || ctx->cfg.read_path == CPT_READ_LINEAR ||
+                   tma_runs(ctx, RasterBatch{members, stride, pitch, n})) {
+            // read in place: the linear kernels take any alignment, tensor maps
+            // 16 bytes (runs: of the members only)
             RasterBatch b{members, stride, pitch, n};
             rc = begin_chunk(ctx);
             if (!rc) rc = accumulate(ctx, b, sign);
         } else {
-            rc = run_staged(ctx, src, n, stride, pitch, sign);
+            rc = run_staged(ctx, src, n, stride, pitch, sign, true);
         }
     } else if (kind == kPinned) {
         const bool aligned = (reinterpret_cast<uintptr_t>(members) % 16 == 0) && (pitch % 16 == 0) && (stride % 16 == 0);
@@ -902,7 +916,6 @@ int composite_begin(composite_ctx **out, int32_t width, int32_t height, const co
         composite_default_config(&c);
     int rc = check_config(c);
     if (rc) return rc;
-    if (c.tma_box_bytes == 0) c.tma_box_bytes = kDefaultTmaBoxBytes;
     composite_ctx *ctx = new composite_ctx();
     ctx->width = width;
     ctx->height = height;

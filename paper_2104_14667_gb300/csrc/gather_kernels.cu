@@ -1,11 +1,17 @@
-// gather_kernels.cu -- the server's overflow upload: a cycle's distinct
-// overflow rasters, scattered over the pinned host part, gathered into one
-// device staging half by a single launch on the copy stream.  The kernel
-// reads host memory through its device mapping over the host link, so one
-// launch replaces one copy call per raster (a cycle moves about a thousand).
+// gather_kernels.cu -- copies into staging memory that a kernel makes better
+// than the copy calls.
+//
+// The server's overflow upload: a cycle's distinct overflow rasters, scattered
+// over the pinned host part, gathered into one device staging half by a single
+// launch on the copy stream.  The kernel reads host memory through its device
+// mapping over the host link, so one launch replaces one copy call per raster
+// (a cycle moves about a thousand).
+//
+// Device rasters at odd pitches or addresses into aligned staging rows, for the
+// paths that need those (tensor maps, float arrays).
 #include <algorithm>
 
-#include "internal.cuh"
+#include "mask_load.cuh"
 
 namespace cpt {
 namespace {
@@ -27,7 +33,49 @@ gather_rasters_kernel(uint8_t *dst, const uint8_t *src, const int32_t *ids, int 
     }
 }
 
+// One 16-byte vector of a staging row per thread and member; blockIdx.y
+// strides over the members.  Bound by HBM: two bytes moved per byte.
+__global__ void __launch_bounds__(kThreads)
+repitch_kernel(uint8_t *dst, int64_t dpitch, int64_t dmember, RasterBatch b, int64_t row, int height, int vecs_per_row) {
+    const int64_t t = blockIdx.x * (int64_t)kThreads + threadIdx.x;
+    if (t >= (int64_t)vecs_per_row * height) return;
+    const int y = (int)(t / vecs_per_row);
+    const int64_t x = (t - (int64_t)y * vecs_per_row) * 16;
+    const int valid = (int)min((int64_t)16, row - x);
+    const uint8_t *base = static_cast<const uint8_t *>(b.base);
+    const uintptr_t lo = reinterpret_cast<uintptr_t>(base);
+    const uintptr_t end = reinterpret_cast<uintptr_t>(batch_end(b, row, height));
+    for (int m = blockIdx.y; m < b.n; m += gridDim.y) {
+        const uint8_t *q = base + (int64_t)m * b.member_stride + (int64_t)y * b.row_pitch + x;
+        const uint32_t shift = (uint32_t)reinterpret_cast<uintptr_t>(q) & 15u;
+        const uintptr_t block = reinterpret_cast<uintptr_t>(q) - shift;
+        uint4 v;
+        if (block >= lo && block + 32 <= end) {
+            const uint4 *at = reinterpret_cast<const uint4 *>(block);
+            v = align_group(__ldg(at), __ldg(at + 1), shift);
+            uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w[i] &= 0xFFu * valid_byte_mask(i, valid);
+            v = make_uint4(w[0], w[1], w[2], w[3]);
+        } else {
+            v = load_group_bytes(q, valid);
+        }
+        *reinterpret_cast<uint4 *>(dst + (int64_t)m * dmember + (int64_t)y * dpitch + x) = v;
+    }
+}
+
 }  // namespace
+
+cudaError_t launch_repitch(void *dst, int64_t dpitch, int64_t dmember, const RasterBatch &b, int64_t row, int height,
+                           cudaStream_t s) {
+    if (b.n <= 0 || row <= 0 || height <= 0) return cudaSuccess;
+    const int vecs = (int)((row + 15) / 16);
+    const int64_t blocks = ((int64_t)vecs * height + kThreads - 1) / kThreads;
+    if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
+    repitch_kernel<<<dim3((unsigned)blocks, (unsigned)std::min(b.n, 65535)), kThreads, 0, s>>>(
+        static_cast<uint8_t *>(dst), dpitch, dmember, b, row, height, vecs);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_gather_rasters(void *dst, const void *src, const int32_t *ids, int n, int64_t stride,
                                   int64_t raster_bytes, const DeviceCaps &caps, cudaStream_t s) {

@@ -65,6 +65,11 @@ cudaError_t launch_pack_to_array(const RasterBatch &b, int width, int height, cu
 // each, i < n; src may be host-mapped pinned memory.  16-byte aligned.
 cudaError_t launch_gather_rasters(void *dst, const void *src, const int32_t *ids, int n, int64_t stride,
                                   int64_t raster_bytes, const DeviceCaps &caps, cudaStream_t s);
+// A batch of rasters of `row` bytes by `height` rows, at any alignment, into
+// rows of dpitch and members of dmember bytes (16-byte aligned, zero past the
+// row): device memory only.
+cudaError_t launch_repitch(void *dst, int64_t dpitch, int64_t dmember, const RasterBatch &b, int64_t row, int height,
+                           cudaStream_t s);
 // Linear rasters (16-byte aligned base, pitch and stride) -> the layers of a
 // cudaArray of 16-byte texels, through a surface object.
 cudaError_t launch_convert_to_array(const void *src, int64_t pitch, int64_t member_stride,
@@ -82,6 +87,12 @@ cudaError_t launch_depth_tma(const CUtensorMap &map, const RasterBatch &b, const
                              int *flags, uint64_t timeout_ns, int box_bytes, const DeviceCaps &caps,
                              cudaStream_t s);
 bool tma_box_supported(int box_bytes);
+// box_bytes of a launch over runs: rasters without row padding as 2 KiB pieces
+// of one run of bytes per member, whatever their width; the map comes from
+// encode_tma_run_map.  tma_run_compatible says whether a batch allows it.
+constexpr int kTmaRuns = 0;
+bool tma_run_compatible(const RasterBatch &b, int width, int height, int elem_bytes);
+int encode_tma_run_map(CUtensorMap *map, const RasterBatch &b, int width, int height, int elem_bytes);
 // Bit-packed masks through cp.async.bulk copies of contiguous 2 KiB pieces
 // into a shared-memory ring (device memory only).  Needs unpadded rows (width
 // a multiple of 32, row pitch width / 8), a 16-byte aligned base and member

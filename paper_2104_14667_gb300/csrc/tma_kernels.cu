@@ -103,11 +103,20 @@ __device__ __forceinline__ void tma_load_box(void *dst, const CUtensorMap *map, 
         : "memory");
 }
 
+__device__ __forceinline__ void tma_load_run(void *dst, const CUtensorMap *map, int x, int z, uint64_t *bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(z), "r"(smem_u32(bar))
+        : "memory");
+}
+
 __device__ __forceinline__ uint4 lds16(const uint8_t *p) {
     return *reinterpret_cast<const uint4 *>(p);
 }
 
-// The producer role: one thread issues every box of the CTA's tiles.
+// The producer role: one thread issues every box of the CTA's tiles (box_rows
+// 0: runs, see kRunBytes).
 __device__ void produce(TmaShared &sh, const CUtensorMap *map, int tiles, int tiles_x,
                         int slabs, int box_x_elems, int box_rows, uint64_t timeout_ns, int *flags) {
     uint32_t it = 0;
@@ -122,8 +131,11 @@ __device__ void produce(TmaShared &sh, const CUtensorMap *map, int tiles, int ti
                 break;
             }
             mbar_arrive_expect_tx(&sh.full[s], kBoxBytes);
-            tma_load_box(sh.stage[s], map, tx * box_x_elems, ty * box_rows, slab * kBoxMembers,
-                         &sh.full[s]);
+            if (box_rows == 0)
+                tma_load_run(sh.stage[s], map, tile * box_x_elems, slab * kBoxMembers, &sh.full[s]);
+            else
+                tma_load_box(sh.stage[s], map, tx * box_x_elems, ty * box_rows, slab * kBoxMembers,
+                             &sh.full[s]);
         }
     }
     if (!ok) {
@@ -138,17 +150,54 @@ __device__ void produce(TmaShared &sh, const CUtensorMap *map, int tiles, int ti
     }
 }
 
+// Runs.  Where a member's rows follow one another without padding, its raster
+// is one run of bytes and a box is 2 KiB of it for 16 members: a 2-D map (byte
+// of the run in 8-byte elements, member), whatever the width.  A box of rows
+// fetches 256-byte pieces a row apart, the widest a box of byte elements can
+// be, and rows that are no multiple of 16 bytes had to be copied first.
+// 4096^2 x 128 masks with clear and render: 371 us by boxes, 364 by runs;
+// unaligned widths 2 to 15 times faster than by way of staging slots.
+constexpr int kRunBytes = kMemberPlaneBytes;
+constexpr int kRunElem = 8;
+
+// 16 counts of pixels i .. i + valid - 1 (in the run's order) folded into a
+// plane whose rows are padded: pixel by pixel, on into the next row.
+template <typename CountT>
+__device__ __forceinline__ void apply_count_run(CountT *plane, int64_t pitch, int width, int64_t i, int valid,
+                                                const uint32_t (&wide)[16], int sign, int *flags) {
+    const int64_t y = i / width;
+    int x = (int)(i - y * width);
+    CountT *row = plane + y * pitch;
+    bool under = false;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        if (j >= valid) break;
+        const uint32_t old = row[x];
+        under |= sign < 0 && wide[j] > old;
+        row[x] = (CountT)(sign > 0 ? old + wide[j] : old - wide[j]);
+        if (++x == width) {
+            x = 0;
+            row += pitch;
+        }
+    }
+    if (under) flag_set(flags, kFlagUnderflow);
+}
+
+// kBoxX = 0: runs.
 template <typename CountT, int kBoxX>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 count_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members, int sign,
                  int *flags, uint64_t timeout_ns) {
-    constexpr int kRows = kMemberPlaneBytes / kBoxX;
-    constexpr int kGroupsPerRow = kBoxX / 16;
+    constexpr bool kRun = kBoxX == 0;
+    constexpr int kWidth = kRun ? kRunBytes : kBoxX;
+    constexpr int kRows = kMemberPlaneBytes / kWidth;
+    constexpr int kGroupsPerRow = kWidth / 16;
     extern __shared__ uint8_t smem_raw[];
     TmaShared &sh = *reinterpret_cast<TmaShared *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
-    const int tiles_x = (p.width + kBoxX - 1) / kBoxX;
-    const int tiles = tiles_x * ((p.height + kRows - 1) / kRows);
+    const int64_t pixels = (int64_t)p.width * p.height;
+    const int tiles_x = kRun ? 1 : (p.width + kWidth - 1) / kWidth;
+    const int tiles = kRun ? (int)((pixels + kRunBytes - 1) / kRunBytes) : tiles_x * ((p.height + kRows - 1) / kRows);
     const int slabs = (n_members + kBoxMembers - 1) / kBoxMembers;
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -162,13 +211,13 @@ count_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members
 
     if (threadIdx.x >= kConsumers) {
         if (threadIdx.x == kConsumers)
-            produce(sh, &map, tiles, tiles_x, slabs, kBoxX, kRows, timeout_ns, flags);
+            produce(sh, &map, tiles, tiles_x, slabs, kRun ? kRunBytes / kRunElem : kBoxX, kRun ? 0 : kRows, timeout_ns, flags);
         return;
     }
 
     CountT *plane = static_cast<CountT *>(p.data);
     const int row = threadIdx.x / kGroupsPerRow, grp = threadIdx.x % kGroupsPerRow;
-    const int offset = row * kBoxX + grp * 16;
+    const int offset = row * kWidth + grp * 16;
     uint32_t it = 0;
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         const int tx = tile % tiles_x, ty = tile / tiles_x;
@@ -202,8 +251,18 @@ count_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members
             }
         }
         widen16(wide, k0, k1, k2, k3);
+        if constexpr (kRun) {
+            const int64_t i = (int64_t)tile * kRunBytes + offset;
+            const int valid = (int)min((int64_t)16, pixels - i);
+            if (valid <= 0) continue;
+            if (p.pitch == p.width)
+                apply_count_group<CountT>(plane + i, 16, wide, sign, flags);
+            else
+                apply_count_run<CountT>(plane, p.pitch, p.width, i, valid, wide, sign, flags);
+            continue;
+        }
         const int y = ty * kRows + row;
-        const int x0 = tx * kBoxX + grp * 16;
+        const int x0 = tx * kWidth + grp * 16;
         if (y < p.height && x0 < p.width)
             apply_count_group<CountT>(plane + (int64_t)y * p.pitch + x0, min(16, p.width - x0),
                                       wide, sign, flags);
@@ -214,14 +273,17 @@ template <int kBoxX>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 depth_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members, int sign,
                  int *flags, uint64_t timeout_ns) {
-    constexpr int kRows = kMemberPlaneBytes / kBoxX;
-    constexpr int kGroupsPerRow = kBoxX / 16;
-    constexpr int kBoxXElems = kBoxX / 4;      // float32 pixels per box row
+    constexpr bool kRun = kBoxX == 0;
+    constexpr int kWidth = kRun ? kRunBytes : kBoxX;
+    constexpr int kRows = kMemberPlaneBytes / kWidth;
+    constexpr int kGroupsPerRow = kWidth / 16;
+    constexpr int kBoxXElems = kWidth / 4;     // float32 pixels per box row
     extern __shared__ uint8_t smem_raw[];
     TmaShared &sh = *reinterpret_cast<TmaShared *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
-    const int tiles_x = (p.width + kBoxXElems - 1) / kBoxXElems;
-    const int tiles = tiles_x * ((p.height + kRows - 1) / kRows);
+    const int64_t pixels = (int64_t)p.width * p.height;
+    const int tiles_x = kRun ? 1 : (p.width + kBoxXElems - 1) / kBoxXElems;
+    const int tiles = kRun ? (int)((pixels + kBoxXElems - 1) / kBoxXElems) : tiles_x * ((p.height + kRows - 1) / kRows);
     const int slabs = (n_members + kBoxMembers - 1) / kBoxMembers;
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -235,17 +297,18 @@ depth_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members
 
     if (threadIdx.x >= kConsumers) {
         if (threadIdx.x == kConsumers)
-            produce(sh, &map, tiles, tiles_x, slabs, kBoxXElems, kRows, timeout_ns, flags);
+            produce(sh, &map, tiles, tiles_x, slabs, kRun ? kRunBytes / kRunElem : kBoxXElems, kRun ? 0 : kRows, timeout_ns,
+                    flags);
         return;
     }
 
     float *plane = static_cast<float *>(p.data);
     const int row = threadIdx.x / kGroupsPerRow, grp = threadIdx.x % kGroupsPerRow;
-    const int offset = row * kBoxX + grp * 16;
+    const int offset = row * kWidth + grp * 16;
     uint32_t it = 0;
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         const int tx = tile % tiles_x, ty = tile / tiles_x;
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        float acc[4] = {0.f, 0.f, 0.f, 0.f}, block[4] = {0.f, 0.f, 0.f, 0.f};
         for (int slab = 0; slab < slabs; ++slab, ++it) {
             const int s = it % kStages;
             if (!wait_bounded(&sh.full[s], (it / kStages) & 1u, timeout_ns, &sh.abort)) {
@@ -254,15 +317,47 @@ depth_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members
                 return;
             }
             const uint8_t *box = sh.stage[s] + offset;
+            // eight members a tree, 64 a block, then the total: as the linear path
 #pragma unroll
-            for (int m = 0; m < kBoxMembers; ++m) {
-                const float4 v = *reinterpret_cast<const float4 *>(box + m * kMemberPlaneBytes);
-                acc[0] += v.x;
-                acc[1] += v.y;
-                acc[2] += v.z;
-                acc[3] += v.w;
+            for (int m = 0; m < kBoxMembers; m += 8) {
+                float4 v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = *reinterpret_cast<const float4 *>(box + (m + j) * kMemberPlaneBytes);
+                block[0] += ((v[0].x + v[1].x) + (v[2].x + v[3].x)) + ((v[4].x + v[5].x) + (v[6].x + v[7].x));
+                block[1] += ((v[0].y + v[1].y) + (v[2].y + v[3].y)) + ((v[4].y + v[5].y) + (v[6].y + v[7].y));
+                block[2] += ((v[0].z + v[1].z) + (v[2].z + v[3].z)) + ((v[4].z + v[5].z) + (v[6].z + v[7].z));
+                block[3] += ((v[0].w + v[1].w) + (v[2].w + v[3].w)) + ((v[4].w + v[5].w) + (v[6].w + v[7].w));
             }
             mbar_arrive(&sh.empty[s]);
+            if (slab % 4 == 3 || slab + 1 == slabs) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    acc[i] += block[i];
+                    block[i] = 0.f;
+                }
+            }
+        }
+        if constexpr (kRun) {
+            const int64_t i = (int64_t)tile * kBoxXElems + grp * 4;
+            const int valid = (int)min((int64_t)4, pixels - i);
+            if (valid <= 0) continue;
+            if (p.pitch == p.width) {
+                apply_depth_group(plane + i, 4, acc, sign);
+            } else {
+                int64_t py = i / p.width;
+                int px = (int)(i - py * p.width);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (j >= valid) break;
+                    float *dst = plane + py * p.pitch + px;
+                    *dst = sign > 0 ? *dst + acc[j] : *dst - acc[j];
+                    if (++px == p.width) {
+                        px = 0;
+                        ++py;
+                    }
+                }
+            }
+            continue;
         }
         const int y = ty * kRows + row;
         const int x0 = tx * kBoxXElems + grp * 4;
@@ -526,6 +621,13 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encoder() {
     return fn;
 }
 
+// Tiles of a plane for boxes of box_bytes by rows, or runs (box_bytes 0).
+int tma_tiles(const Plane &p, int elem_bytes, int box_bytes) {
+    if (box_bytes == 0) return (int)(((int64_t)p.width * p.height * elem_bytes + kRunBytes - 1) / kRunBytes);
+    const int box_px = box_bytes / elem_bytes, rows = kMemberPlaneBytes / box_bytes;
+    return ((p.width + box_px - 1) / box_px) * ((p.height + rows - 1) / rows);
+}
+
 unsigned grid_for(int tiles, const DeviceCaps &caps) {
     const int cap = caps.num_sms * kCtasPerSm;
     return (unsigned)(tiles < cap ? tiles : cap);
@@ -560,13 +662,32 @@ int encode_tma_map(CUtensorMap *map, const RasterBatch &b, int width, int height
     return (int)r;
 }
 
+bool tma_run_compatible(const RasterBatch &b, int width, int height, int elem_bytes) {
+    const int64_t bytes = (int64_t)width * height * elem_bytes;
+    // tiles are numbered in 32 bits, the run's 8-byte elements too
+    return b.row_pitch == (int64_t)width * elem_bytes && bytes % 16 == 0 && b.member_stride % 16 == 0 &&
+           reinterpret_cast<uintptr_t>(b.base) % 16 == 0 && bytes / kRunElem <= INT32_MAX;
+}
+
+int encode_tma_run_map(CUtensorMap *map, const RasterBatch &b, int width, int height, int elem_bytes) {
+    PFN_cuTensorMapEncodeTiled_v12000 enc = get_encoder();
+    if (!enc) return CUDA_ERROR_NOT_FOUND;
+    if (!tma_run_compatible(b, width, height, elem_bytes)) return CUDA_ERROR_INVALID_VALUE;
+    cuuint64_t dims[2] = {(cuuint64_t)width * height * elem_bytes / kRunElem, (cuuint64_t)b.n};
+    cuuint64_t strides[1] = {(cuuint64_t)b.member_stride};
+    cuuint32_t box[2] = {kRunBytes / kRunElem, kBoxMembers};
+    cuuint32_t estrides[2] = {1, 1};
+    return (int)enc(map, CU_TENSOR_MAP_DATA_TYPE_INT64, 2, const_cast<void *>(b.base), dims, strides, box, estrides,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+}
+
 template <typename CountT, int kBoxX>
 cudaError_t launch_count_tma_t(const CUtensorMap &map, const RasterBatch &b, const Plane &p, int sign,
                                int *flags, uint64_t timeout_ns, const DeviceCaps &caps, cudaStream_t s) {
-    constexpr int kRows = kMemberPlaneBytes / kBoxX;
     const cudaError_t prep = allow_smem(reinterpret_cast<const void *>(count_tma_kernel<CountT, kBoxX>), kSmemBytes);
     if (prep != cudaSuccess) return prep;
-    const int tiles = ((p.width + kBoxX - 1) / kBoxX) * ((p.height + kRows - 1) / kRows);
+    const int tiles = tma_tiles(p, 1, kBoxX);
     count_tma_kernel<CountT, kBoxX><<<grid_for(tiles, caps), kThreads, kSmemBytes, s>>>(
         map, p, b.n, sign, flags, timeout_ns);
     return cudaGetLastError();
@@ -575,10 +696,9 @@ cudaError_t launch_count_tma_t(const CUtensorMap &map, const RasterBatch &b, con
 template <int kBoxX>
 cudaError_t launch_depth_tma_t(const CUtensorMap &map, const RasterBatch &b, const Plane &p, int sign,
                                int *flags, uint64_t timeout_ns, const DeviceCaps &caps, cudaStream_t s) {
-    constexpr int kRows = kMemberPlaneBytes / kBoxX;
     const cudaError_t prep = allow_smem(reinterpret_cast<const void *>(depth_tma_kernel<kBoxX>), kSmemBytes);
     if (prep != cudaSuccess) return prep;
-    const int tiles = ((p.width + kBoxX / 4 - 1) / (kBoxX / 4)) * ((p.height + kRows - 1) / kRows);
+    const int tiles = tma_tiles(p, 4, kBoxX);
     depth_tma_kernel<kBoxX><<<grid_for(tiles, caps), kThreads, kSmemBytes, s>>>(map, p, b.n, sign, flags,
                                                                                  timeout_ns);
     return cudaGetLastError();
@@ -590,6 +710,9 @@ cudaError_t launch_count_tma(const CUtensorMap &map, const RasterBatch &b, const
     if (b.n <= 0) return cudaSuccess;
     const bool u16 = p.count_bits == 16;
     switch (box_bytes) {
+        case kTmaRuns:
+            return u16 ? launch_count_tma_t<uint16_t, 0>(map, b, p, sign, flags, timeout_ns, caps, s)
+                       : launch_count_tma_t<uint32_t, 0>(map, b, p, sign, flags, timeout_ns, caps, s);
         case 64:
             return u16 ? launch_count_tma_t<uint16_t, 64>(map, b, p, sign, flags, timeout_ns, caps, s)
                        : launch_count_tma_t<uint32_t, 64>(map, b, p, sign, flags, timeout_ns, caps, s);
@@ -651,6 +774,7 @@ cudaError_t launch_depth_tma(const CUtensorMap &map, const RasterBatch &b, const
                              cudaStream_t s) {
     if (b.n <= 0) return cudaSuccess;
     switch (box_bytes) {
+        case kTmaRuns: return launch_depth_tma_t<0>(map, b, p, sign, flags, timeout_ns, caps, s);
         case 64: return launch_depth_tma_t<64>(map, b, p, sign, flags, timeout_ns, caps, s);
         case 128: return launch_depth_tma_t<128>(map, b, p, sign, flags, timeout_ns, caps, s);
         case 256: return launch_depth_tma_t<256>(map, b, p, sign, flags, timeout_ns, caps, s);
