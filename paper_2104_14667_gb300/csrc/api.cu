@@ -478,31 +478,58 @@ int convert_to_array(composite_ctx *ctx, Slot &s, const RasterBatch &b, cudaStre
     return trace_close(ctx, st);
 }
 
-// Consumes one staged chunk on the compute stream.
-int consume_slot(composite_ctx *ctx, Slot &s, int c, int sign) {
-    RasterBatch b{s.stage, ctx->member_bytes, ctx->stage_pitch, c};
+// Consumes one staged chunk, the rasters of b in slot s, on the compute stream.
+int consume_slot(composite_ctx *ctx, Slot &s, const RasterBatch &b, int sign) {
     if (ctx->cfg.read_path == CPT_READ_TEXTURE) {
         int rc = convert_to_array(ctx, s, b, ctx->compute);
         if (rc) return rc;
-        return accumulate_texture(ctx, s, c, sign);
+        return accumulate_texture(ctx, s, b.n, sign);
     }
     return accumulate(ctx, b, sign);
 }
 
+// The rasters of a slot as the uploads lay them out: rows of stage_pitch bytes.
+RasterBatch staged_batch(const composite_ctx *ctx, const Slot &s, int c) {
+    return RasterBatch{s.stage, ctx->member_bytes, ctx->stage_pitch, c};
+}
+
+// Whether c host rasters may be uploaded as the one run of bytes that they
+// are, row padding included, and read from the slot at their own pitch: their
+// rows follow one another within a slot's bytes, and the path reads any
+// alignment (the tensor maps: where they are runs).  A pitched copy moves row
+// by row: 506 x 4482 x 116 masks took 18 ms that way, 15 GB/s of a link of 210.
+bool upload_as_one(const composite_ctx *ctx, const Slot &s, int64_t stride, int64_t pitch, int c) {
+    if (stride != pitch * ctx->height || pitch > ctx->stage_pitch) return false;
+    if (ctx->cfg.read_path == CPT_READ_LINEAR) return true;
+    if (ctx->cfg.read_path == CPT_READ_TEXTURE) return ctx->packed_array;
+    return tma_runs(ctx, RasterBatch{s.stage, stride, pitch, c});
+}
+
 // Uploads c rasters (pinned host or device memory) into a staging buffer laid
-// out with row pitch stage_pitch and raster stride member_bytes.  Device
-// rasters go by a kernel: as pitched copies, 154-pixel depth rows moved at
-// 1 TB/s.
+// out with row pitch stage_pitch and raster stride member_bytes: one copy where
+// the layouts agree; pitched copies where pinned rows start on 16-byte
+// boundaries (190-200 GB/s); else a kernel that moves the rows (pinned rasters
+// through their device mapping, over the host link, at 170-180 GB/s), since
+// pitched copies of rows 506 and 3164 bytes apart went at 15 and 58 GB/s, and
+// device rows of 154 floats at 1 TB/s.
 int upload(composite_ctx *ctx, uint8_t *dst, const uint8_t *src, int c, int64_t stride,
            int64_t pitch, bool device) {
     const int64_t row = ctx->row_bytes;
     const int64_t dpitch = ctx->stage_pitch;
     const int64_t h = ctx->height;
-    if (device) {
-        CK(ctx, cpt::launch_repitch(dst, dpitch, ctx->member_bytes, RasterBatch{src, stride, pitch, c}, row, ctx->height,
-                                    ctx->copy));
-    } else if (pitch == row && row == dpitch && stride == pitch * h) {
+    if (pitch == row && row == dpitch && stride == pitch * h) {
         CK(ctx, cudaMemcpyAsync(dst, src, (size_t)c * ctx->member_bytes, cudaMemcpyDefault, ctx->copy));
+        return CPT_OK;
+    }
+    void *mapped = nullptr;
+    const bool aligned = (reinterpret_cast<uintptr_t>(src) | (uintptr_t)pitch | (uintptr_t)stride) % 16 == 0;
+    if (!device && !aligned && cudaHostGetDevicePointer(&mapped, const_cast<uint8_t *>(src), 0) != cudaSuccess) {
+        cudaGetLastError();
+        mapped = nullptr;
+    }
+    if (device || mapped) {
+        const RasterBatch b{device ? src : mapped, stride, pitch, c};
+        CK(ctx, cpt::launch_repitch(dst, dpitch, ctx->member_bytes, b, row, ctx->height, ctx->copy));
     } else if (stride == pitch * h) {
         CK(ctx, cudaMemcpy2DAsync(dst, dpitch, src, pitch, row, (size_t)c * h, cudaMemcpyDefault, ctx->copy));
     } else {
@@ -541,13 +568,21 @@ int run_staged(composite_ctx *ctx, const uint8_t *src, int n, int64_t stride, in
         CK(ctx, cudaStreamWaitEvent(ctx->copy, s.consumed, 0));
         rc = trace_open(ctx, kTraceUpload, ctx->copy);
         if (rc) return rc;
-        rc = upload(ctx, s.stage, src + (int64_t)m0 * stride, c, stride, pitch, device);
-        if (rc) return rc;
+        RasterBatch b = staged_batch(ctx, s, c);
+        if (!device && upload_as_one(ctx, s, stride, pitch, c)) {
+            b.member_stride = stride;
+            b.row_pitch = pitch;
+            const int64_t bytes = (c - 1) * stride + (ctx->height - 1) * pitch + ctx->row_bytes;
+            CK(ctx, cudaMemcpyAsync(s.stage, src + (int64_t)m0 * stride, (size_t)bytes, cudaMemcpyDefault, ctx->copy));
+        } else {
+            rc = upload(ctx, s.stage, src + (int64_t)m0 * stride, c, stride, pitch, device);
+            if (rc) return rc;
+        }
         rc = trace_close(ctx, ctx->copy);
         if (rc) return rc;
         CK(ctx, cudaEventRecord(s.ready, ctx->copy));
         CK(ctx, cudaStreamWaitEvent(ctx->compute, s.ready, 0));
-        rc = consume_slot(ctx, s, c, sign);
+        rc = consume_slot(ctx, s, b, sign);
         if (rc) return rc;
         CK(ctx, cudaEventRecord(s.consumed, ctx->compute));
     }
@@ -688,7 +723,7 @@ int run_ring(composite_ctx *ctx, const uint8_t *src, int n, int64_t stride, int6
         CK(ctx, cudaEventRecord(s.ready, ctx->copy));
         s.ring_used = true;
         CK(ctx, cudaStreamWaitEvent(ctx->compute, s.ready, 0));
-        rc = consume_slot(ctx, s, c, sign);
+        rc = consume_slot(ctx, s, staged_batch(ctx, s, c), sign);
         if (rc) return rc;
         CK(ctx, cudaEventRecord(s.consumed, ctx->compute));
     }
