@@ -751,16 +751,18 @@ int composite_server_drain(composite_server *s) try {
     s->err.clear();
     auto deadline = std::chrono::steady_clock::now() + std::chrono::milliseconds(timeout_ms(s));
     int64_t last_done = s->stats.requests_done;
-    for (unsigned spin = 0; s->stats.queued > 0 || s->stats.in_flight > 0; ++spin) {
+    cpt::PollPause pause;
+    while (s->stats.queued > 0 || s->stats.in_flight > 0) {
         int rc = composite_server_pump(s, nullptr, 0, nullptr);
         if (rc) return rc;
         if (s->stats.requests_done != last_done) {
             last_done = s->stats.requests_done;
             deadline = std::chrono::steady_clock::now() + std::chrono::milliseconds(timeout_ms(s));
+            pause = cpt::PollPause();
         } else if (std::chrono::steady_clock::now() > deadline) {
             return sfail(s, CPT_ETIMEOUT, "no request completed within %lld ms", (long long)timeout_ms(s));
         }
-        if (spin > 200) std::this_thread::sleep_for(std::chrono::microseconds(50));
+        pause();
     }
     return CPT_OK;
 } catch (...) {
