@@ -5,6 +5,7 @@
 
 #include "bit_count.cuh"
 #include "mask_load.cuh"
+#include "overlap.cuh"
 
 namespace cpt {
 namespace {
@@ -39,6 +40,7 @@ count_bits_kernel(RasterBatch b, Plane p, int sign, int *flags, int64_t units, i
     const int64_t stride = b.member_stride;
     const uint8_t *base = static_cast<const uint8_t *>(b.base);
     const uint8_t *end = batch_end(b, (p.width + 7) / 8, p.height);
+    await_previous();
     for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < units * slabs;
          u += (int64_t)gridDim.x * blockDim.x) {
         const int sl = (int)(u / units);
@@ -118,11 +120,11 @@ template <typename CountT>
 void launch_count_bits_t(int loads, unsigned grid, cudaStream_t s, const RasterBatch &b, const Plane &p, int sign, int *flags,
                          int64_t units, int per_row, int slab, int slabs) {
     if (loads == kPairs)
-        count_bits_kernel<CountT, kPairs><<<grid, kThreads, 0, s>>>(b, p, sign, flags, units, per_row, slab, slabs);
+        launch_overlapped(count_bits_kernel<CountT, kPairs>, grid, kThreads, 0, s, b, p, sign, flags, units, per_row, slab, slabs);
     else if (loads == kSingles)
-        count_bits_kernel<CountT, kSingles><<<grid, kThreads, 0, s>>>(b, p, sign, flags, units, per_row, slab, slabs);
+        launch_overlapped(count_bits_kernel<CountT, kSingles>, grid, kThreads, 0, s, b, p, sign, flags, units, per_row, slab, slabs);
     else
-        count_bits_kernel<CountT, kShifted><<<grid, kThreads, 0, s>>>(b, p, sign, flags, units, per_row, slab, slabs);
+        launch_overlapped(count_bits_kernel<CountT, kShifted>, grid, kThreads, 0, s, b, p, sign, flags, units, per_row, slab, slabs);
 }
 
 inline int64_t blocks_for(int64_t groups) {

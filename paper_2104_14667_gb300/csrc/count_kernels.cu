@@ -16,6 +16,7 @@
 #include <algorithm>
 
 #include "mask_load.cuh"
+#include "overlap.cuh"
 
 namespace cpt {
 namespace {
@@ -147,6 +148,7 @@ depth_linear_kernel(RasterBatch b, Plane p, int sign, int64_t groups, int groups
     const int64_t g = (int64_t)blockIdx.x * kGroups + lane_group;
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
     int y = 0, x0 = 0, valid = 0;
+    await_previous();
     if (g < groups) {
         y = (int)(g / groups_per_row);
         x0 = (int)(g - (int64_t)y * groups_per_row) * 4;
@@ -244,10 +246,10 @@ cudaError_t launch_count_t(const RasterBatch &b, const Plane &p, int sign, int *
     if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
     const dim3 grid((unsigned)blocks, (unsigned)c.slabs);
     switch (c.slices) {
-        case 1: count_linear_kernel<CountT, kAligned, 1><<<grid, kThreads, 0, s>>>(b, p, sign, flags, groups, gpr, c.slab); break;
-        case 2: count_linear_kernel<CountT, kAligned, 2><<<grid, kThreads, 0, s>>>(b, p, sign, flags, groups, gpr, c.slab); break;
-        case 4: count_linear_kernel<CountT, kAligned, 4><<<grid, kThreads, 0, s>>>(b, p, sign, flags, groups, gpr, c.slab); break;
-        default: count_linear_kernel<CountT, kAligned, 8><<<grid, kThreads, 0, s>>>(b, p, sign, flags, groups, gpr, c.slab); break;
+        case 1: launch_overlapped(count_linear_kernel<CountT, kAligned, 1>, grid, kThreads, 0, s, b, p, sign, flags, groups, gpr, c.slab); break;
+        case 2: launch_overlapped(count_linear_kernel<CountT, kAligned, 2>, grid, kThreads, 0, s, b, p, sign, flags, groups, gpr, c.slab); break;
+        case 4: launch_overlapped(count_linear_kernel<CountT, kAligned, 4>, grid, kThreads, 0, s, b, p, sign, flags, groups, gpr, c.slab); break;
+        default: launch_overlapped(count_linear_kernel<CountT, kAligned, 8>, grid, kThreads, 0, s, b, p, sign, flags, groups, gpr, c.slab); break;
     }
     return cudaGetLastError();
 }
@@ -262,10 +264,10 @@ cudaError_t launch_depth_t(const RasterBatch &b, const Plane &p, int sign, const
     if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
     const unsigned grid = (unsigned)blocks;
     switch (slices) {
-        case 1: depth_linear_kernel<kAligned, 1><<<grid, kThreads, 0, s>>>(b, p, sign, groups, gpr); break;
-        case 2: depth_linear_kernel<kAligned, 2><<<grid, kThreads, 0, s>>>(b, p, sign, groups, gpr); break;
-        case 4: depth_linear_kernel<kAligned, 4><<<grid, kThreads, 0, s>>>(b, p, sign, groups, gpr); break;
-        default: depth_linear_kernel<kAligned, 8><<<grid, kThreads, 0, s>>>(b, p, sign, groups, gpr); break;
+        case 1: launch_overlapped(depth_linear_kernel<kAligned, 1>, grid, kThreads, 0, s, b, p, sign, groups, gpr); break;
+        case 2: launch_overlapped(depth_linear_kernel<kAligned, 2>, grid, kThreads, 0, s, b, p, sign, groups, gpr); break;
+        case 4: launch_overlapped(depth_linear_kernel<kAligned, 4>, grid, kThreads, 0, s, b, p, sign, groups, gpr); break;
+        default: launch_overlapped(depth_linear_kernel<kAligned, 8>, grid, kThreads, 0, s, b, p, sign, groups, gpr); break;
     }
     return cudaGetLastError();
 }
@@ -273,6 +275,7 @@ cudaError_t launch_depth_t(const RasterBatch &b, const Plane &p, int sign, const
 // Counts (or sums) and device flags to zero, in one launch.
 __global__ void __launch_bounds__(kThreads)
 clear_plane_kernel(uint4 *data, int64_t words, int *flags) {
+    await_previous();
     if (blockIdx.x == 0 && threadIdx.x < kFlagCount) flags[threadIdx.x] = 0;
     for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < words; i += (int64_t)gridDim.x * kThreads)
         data[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -283,7 +286,7 @@ clear_plane_kernel(uint4 *data, int64_t words, int *flags) {
 cudaError_t launch_clear_plane(void *data, int64_t bytes, int *flags, const DeviceCaps &caps, cudaStream_t s) {
     const int64_t words = bytes / 16;   // plane rows are whole 16-byte vectors
     const int64_t blocks = std::min<int64_t>((words + 4 * kThreads - 1) / (4 * kThreads), 8ll * caps.num_sms);
-    clear_plane_kernel<<<(unsigned)std::max<int64_t>(1, blocks), kThreads, 0, s>>>(static_cast<uint4 *>(data), words, flags);
+    launch_overlapped(clear_plane_kernel, (unsigned)std::max<int64_t>(1, blocks), kThreads, 0, s, static_cast<uint4 *>(data), words, flags);
     return cudaGetLastError();
 }
 

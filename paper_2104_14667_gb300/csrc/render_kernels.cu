@@ -5,6 +5,7 @@
 // (render_units.cuh).
 #include <algorithm>
 
+#include "overlap.cuh"
 #include "render_units.cuh"
 
 namespace cpt {
@@ -35,6 +36,7 @@ render_counts_kernel(Plane p, ClassDivisor div, CountT *counts_out, uint8_t *buc
         for (int i = threadIdx.x; i < kWarps * kHistWarpBytes / 16; i += blockDim.x)
             reinterpret_cast<uint4 *>(s_hist)[i] = make_uint4(0, 0, 0, 0);
     __syncthreads();
+    await_previous();
     const CountT *plane = static_cast<const CountT *>(p.data);
     const int64_t total = (int64_t)p.width * p.height;
     constexpr int kItemPixels = 32 * kUnits * 4;
@@ -80,6 +82,7 @@ render_mean_kernel(Plane p, uint64_t n_members, float *mean_out, int vec) {
     const float n = (float)n_members;
     constexpr int kItemPixels = 32 * kUnits * 4;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    await_previous();
     for (int64_t base = ((int64_t)blockIdx.x * kWarps + warp) * kItemPixels; base < total;
          base += (int64_t)gridDim.x * kWarps * kItemPixels) {
         const int left = (int)min(total - base, (int64_t)kItemPixels);
@@ -124,16 +127,13 @@ void launch_counts(const Plane &p, const ClassDivisor &div, CountT *counts_out, 
     const unsigned grid = grid_for((int64_t)p.width * p.height, kUnits, kHist ? kHistCtasPerSm : kCtasPerSm, caps);
     switch (plane_rows(p.pitch, p.width)) {
         case kRowsDense:
-            render_counts_kernel<CountT, kRowsDense, kHist, kUnits><<<grid, kThreads, 0, s>>>(
-                p, div, counts_out, bucket_out, rgba_out, vec, lut, hist_out);
+            launch_overlapped(render_counts_kernel<CountT, kRowsDense, kHist, kUnits>, grid, kThreads, 0, s, p, div, counts_out, bucket_out, rgba_out, vec, lut, hist_out);
             break;
         case kRowsOfFours:
-            render_counts_kernel<CountT, kRowsOfFours, kHist, kUnits><<<grid, kThreads, 0, s>>>(
-                p, div, counts_out, bucket_out, rgba_out, vec, lut, hist_out);
+            launch_overlapped(render_counts_kernel<CountT, kRowsOfFours, kHist, kUnits>, grid, kThreads, 0, s, p, div, counts_out, bucket_out, rgba_out, vec, lut, hist_out);
             break;
         default:
-            render_counts_kernel<CountT, kRowsRagged, kHist, kUnits><<<grid, kThreads, 0, s>>>(
-                p, div, counts_out, bucket_out, rgba_out, vec, lut, hist_out);
+            launch_overlapped(render_counts_kernel<CountT, kRowsRagged, kHist, kUnits>, grid, kThreads, 0, s, p, div, counts_out, bucket_out, rgba_out, vec, lut, hist_out);
     }
 }
 
@@ -156,9 +156,9 @@ template <int kUnits>
 void launch_mean(const Plane &p, uint64_t n_members, float *mean_out, int vec, const DeviceCaps &caps, cudaStream_t s) {
     const unsigned grid = grid_for((int64_t)p.width * p.height, kUnits, kCtasPerSm, caps);
     switch (plane_rows(p.pitch, p.width)) {
-        case kRowsDense: render_mean_kernel<kRowsDense, kUnits><<<grid, kThreads, 0, s>>>(p, n_members, mean_out, vec); break;
-        case kRowsOfFours: render_mean_kernel<kRowsOfFours, kUnits><<<grid, kThreads, 0, s>>>(p, n_members, mean_out, vec); break;
-        default: render_mean_kernel<kRowsRagged, kUnits><<<grid, kThreads, 0, s>>>(p, n_members, mean_out, vec);
+        case kRowsDense: launch_overlapped(render_mean_kernel<kRowsDense, kUnits>, grid, kThreads, 0, s, p, n_members, mean_out, vec); break;
+        case kRowsOfFours: launch_overlapped(render_mean_kernel<kRowsOfFours, kUnits>, grid, kThreads, 0, s, p, n_members, mean_out, vec); break;
+        default: launch_overlapped(render_mean_kernel<kRowsRagged, kUnits>, grid, kThreads, 0, s, p, n_members, mean_out, vec);
     }
 }
 

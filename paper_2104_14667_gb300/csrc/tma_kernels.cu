@@ -19,6 +19,7 @@
 #include <cudaTypedefs.h>
 
 #include "bit_count.cuh"
+#include "overlap.cuh"
 
 namespace cpt {
 namespace {
@@ -208,6 +209,7 @@ count_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    await_previous();
 
     if (threadIdx.x >= kConsumers) {
         if (threadIdx.x == kConsumers)
@@ -294,6 +296,7 @@ depth_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    await_previous();
 
     if (threadIdx.x >= kConsumers) {
         if (threadIdx.x == kConsumers)
@@ -502,6 +505,7 @@ count_bits_bulk_kernel(BitsWork w, Plane p, int sign, int *flags, uint64_t timeo
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    await_previous();
 
     if (threadIdx.x >= kBitsConsumers) {
         produce_bits(sh, w, timeout_ns, flags);
@@ -688,8 +692,7 @@ cudaError_t launch_count_tma_t(const CUtensorMap &map, const RasterBatch &b, con
     const cudaError_t prep = allow_smem(reinterpret_cast<const void *>(count_tma_kernel<CountT, kBoxX>), kSmemBytes);
     if (prep != cudaSuccess) return prep;
     const int tiles = tma_tiles(p, 1, kBoxX);
-    count_tma_kernel<CountT, kBoxX><<<grid_for(tiles, caps), kThreads, kSmemBytes, s>>>(
-        map, p, b.n, sign, flags, timeout_ns);
+    launch_overlapped(count_tma_kernel<CountT, kBoxX>, grid_for(tiles, caps), kThreads, kSmemBytes, s, map, p, b.n, sign, flags, timeout_ns);
     return cudaGetLastError();
 }
 
@@ -699,7 +702,7 @@ cudaError_t launch_depth_tma_t(const CUtensorMap &map, const RasterBatch &b, con
     const cudaError_t prep = allow_smem(reinterpret_cast<const void *>(depth_tma_kernel<kBoxX>), kSmemBytes);
     if (prep != cudaSuccess) return prep;
     const int tiles = tma_tiles(p, 4, kBoxX);
-    depth_tma_kernel<kBoxX><<<grid_for(tiles, caps), kThreads, kSmemBytes, s>>>(map, p, b.n, sign, flags,
+    launch_overlapped(depth_tma_kernel<kBoxX>, grid_for(tiles, caps), kThreads, kSmemBytes, s, map, p, b.n, sign, flags,
                                                                                  timeout_ns);
     return cudaGetLastError();
 }
@@ -737,7 +740,7 @@ cudaError_t launch_bits_bulk_t(const BitsWork &w, unsigned grid, const Plane &p,
                                uint64_t timeout_ns, cudaStream_t s) {
     const cudaError_t prep = allow_smem(reinterpret_cast<const void *>(count_bits_bulk_kernel<CountT>), kBitsSmemBytes);
     if (prep != cudaSuccess) return prep;
-    count_bits_bulk_kernel<CountT><<<grid, kBitsThreads, kBitsSmemBytes, s>>>(w, p, sign, flags, timeout_ns);
+    launch_overlapped(count_bits_bulk_kernel<CountT>, grid, kBitsThreads, kBitsSmemBytes, s, w, p, sign, flags, timeout_ns);
     return cudaGetLastError();
 }
 
