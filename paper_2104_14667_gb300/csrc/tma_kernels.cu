@@ -375,7 +375,7 @@ depth_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members
 // member's raster is one run of 32-pixel words, so a tile of kBitsTileWords
 // consecutive words is one contiguous 2 KiB piece of every member.  The
 // producer warp streams the pieces of 16 members per stage with cp.async.bulk
-// (no tensor map: one lane per member) into a ring of seven 32 KiB
+// (no tensor map: one lane per member) into a ring of six 32 KiB
 // shared-memory stages; four consumer warps keep the counts of 128 pixels per
 // thread in carry-save accumulators, four independent chains per thread.
 // The bytes in flight wait in shared memory instead of registers, which is
@@ -384,6 +384,11 @@ depth_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members
 // ring, 0.367 with 224 KiB, 0.398 with 128 KiB; 8 x 64 0.378; 16 x 64
 // 0.404; 4 x 64 (1 KiB pieces) 0.613; two or three CTAs per SM with smaller
 // rings 0.403.
+// A slab's counts leave through shared memory, so that consecutive threads
+// update consecutive words of the composite: from the threads that hold them
+// every atomic of a warp touched 32 sectors, 256 bytes apart (1856 x 2208 x
+// 1024 with five slabs: 100 us, 95 this way, 5.5 TB/s).  The 33 KB come from
+// the ring: six stages, 192 KiB.
 // Work items are (tile, member slab).  They are numbered in blocks of one
 // tile per CTA, slab after slab within a block, and dealt to the persistent
 // CTAs round robin, so CTA c takes tile c of the block through all its slabs
@@ -391,7 +396,9 @@ depth_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members
 // counts stay in L2 between its slabs.  (Slab-major numbering streamed the
 // whole mask set between two visits of a tile and re-read the count plane
 // from DRAM once per slab; tile-major numbering had up to 18 CTAs folding
-// atomics into the same tile.)  A slab is at most 15 stages (240 members):
+// atomics into the same tile; equal runs of stages for every CTA in the last,
+// partial block balanced 251 tiles on 152 CTAs but took the CTAs to different
+// members at a time: 105 -> 125 us for the pass, and 46 -> 104 for a smaller.)  A slab is at most 15 stages (240 members):
 // the counters hold 255.
 constexpr int kBitsConsumerWarps = 4;
 constexpr int kBitsWordsPerThread = 4;
@@ -401,7 +408,7 @@ constexpr int kBitsTileWords = kBitsConsumers * kBitsWordsPerThread;
 constexpr int kBitsTileBytes = kBitsTileWords * 4;
 constexpr int kBitsStageMembers = 16;
 constexpr int kBitsStageBytes = kBitsTileBytes * kBitsStageMembers;
-constexpr int kBitsRingBytes = 224 * 1024;
+constexpr int kBitsRingBytes = 192 * 1024;
 constexpr int kBitsStages = kBitsRingBytes / kBitsStageBytes;
 constexpr int kBitsCtasPerSm = 1;
 constexpr int kBitsSlabStages = 15;
@@ -411,6 +418,9 @@ static_assert(kBitsWordsPerThread == 1 || kBitsWordsPerThread == 2 || kBitsWords
 
 struct alignas(128) BitsShared {
     uint8_t stage[kBitsStages][kBitsStageBytes];
+    // a slab's counts, two to a word, [word of the thread][thread]: the pad
+    // keeps both orders of access off shared banks
+    uint32_t counts[16 * kBitsWordsPerThread][kBitsConsumers + 1];
     uint64_t full[kBitsStages];
     uint64_t empty[kBitsStages];
     int abort;
@@ -447,6 +457,76 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
             smem_u32(dst)),
         "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(smem_u32(bar))
         : "memory");
+}
+
+// Barriers of the consumer warps alone.  Every consumer thread reaches them:
+// the waits before them are bounded, and a warp whose wait ran out goes on to
+// the barrier, where all learn of it at once and leave together.
+__device__ __forceinline__ void consumers_sync() {
+    asm volatile("bar.sync 1, %0;" ::"n"(kBitsConsumers) : "memory");
+}
+
+__device__ __forceinline__ bool consumers_any(bool x) {
+    uint32_t any;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 q, %1, 0;\n\t"
+        "bar.red.or.pred p, 1, %2, q;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(any)
+        : "r"((uint32_t)x), "n"(kBitsConsumers)
+        : "memory");
+    return any != 0;
+}
+
+// Two neighbouring counts, the first of them at an even pixel: loaded, stored
+// with d's halves added or taken away, or updated by atomics; true when a
+// subtraction went below zero.
+template <typename CountT>
+__device__ __forceinline__ void load_pair(const CountT *p, uint32_t (&old)[2]) {
+    if constexpr (sizeof(CountT) == 2) {
+        const uint32_t v = *reinterpret_cast<const uint32_t *>(p);
+        old[0] = v & 0xFFFFu, old[1] = v >> 16;
+    } else {
+        const uint2 v = *reinterpret_cast<const uint2 *>(p);
+        old[0] = v.x, old[1] = v.y;
+    }
+}
+
+template <typename CountT>
+__device__ __forceinline__ bool store_pair(CountT *p, const uint32_t (&old)[2], uint32_t d, int sign) {
+    const uint32_t d0 = d & 0xFFFFu, d1 = d >> 16;
+    const uint32_t c0 = sign > 0 ? old[0] + d0 : old[0] - d0, c1 = sign > 0 ? old[1] + d1 : old[1] - d1;
+    if constexpr (sizeof(CountT) == 2)
+        *reinterpret_cast<uint32_t *>(p) = (c0 & 0xFFFFu) | (c1 << 16);
+    else
+        *reinterpret_cast<uint2 *>(p) = make_uint2(c0, c1);
+    return sign < 0 && (d0 > old[0] || d1 > old[1]);
+}
+
+template <typename CountT>
+__device__ __forceinline__ bool atomic_pair(CountT *p, uint32_t d, int sign) {
+    if (d == 0) return false;
+    uint32_t *w = reinterpret_cast<uint32_t *>(p);
+    const uint32_t d0 = d & 0xFFFFu, d1 = d >> 16;
+    if constexpr (sizeof(CountT) == 2) {
+        if (sign > 0) {
+            atomicAdd(w, d);
+            return false;
+        }
+        const uint32_t old = atomicSub(w, d);
+        return d0 > (old & 0xFFFFu) || d1 > (old >> 16);
+    } else {
+        if (sign > 0) {
+            if (d0) atomicAdd(w, d0);
+            if (d1) atomicAdd(w + 1, d1);
+            return false;
+        }
+        bool under = false;
+        if (d0) under |= d0 > atomicSub(w, d0);
+        if (d1) under |= d1 > atomicSub(w + 1, d1);
+        return under;
+    }
 }
 
 // The producer warp: lane 0 waits for a free stage and announces its bytes,
@@ -521,13 +601,15 @@ count_bits_bulk_kernel(BitsWork w, Plane p, int sign, int *flags, uint64_t timeo
         const int m0 = slab * w.slab_stages * kBitsStageMembers;
         const int m1 = min(w.n, m0 + w.slab_stages * kBitsStageMembers);
         BitCounter acc[kBitsWordsPerThread];
+        bool failed = false;
         for (int ms = m0; ms < m1; ms += kBitsStageMembers, ++it) {
             const int s = it % kBitsStages;
             const int cnt = min(kBitsStageMembers, m1 - ms);
-            if (!wait_bounded(&sh.full[s], (it / kBitsStages) & 1u, timeout_ns, &sh.abort)) {
+            if (!__all_sync(0xFFFFFFFFu, wait_bounded(&sh.full[s], (it / kBitsStages) & 1u, timeout_ns, &sh.abort))) {
                 flag_set(flags, kFlagTimeout);
                 sh.abort = 1;
-                return;
+                failed = true;
+                break;   // the whole warp
             }
             const uint8_t *src = sh.stage[s] + 4 * kBitsWordsPerThread * tid;
             uint32_t wv[kBitsWordsPerThread][16];
@@ -554,25 +636,44 @@ count_bits_bulk_kernel(BitsWork w, Plane p, int sign, int *flags, uint64_t timeo
             __syncwarp();
             if ((tid & 31) == 0) mbar_arrive(&sh.empty[s]);
         }
-        // words past the raster's last (a partial tile) hold stale bytes and are skipped
-        const int64_t word0 = (int64_t)tile * kBitsTileWords + kBitsWordsPerThread * tid;
 #pragma unroll
         for (int j = 0; j < kBitsWordsPerThread; ++j) {
-            const int64_t g = word0 + j;
-            if (g >= w.words) break;
-            const int y = (int)(g / w.words_per_row);
-            const int x0 = 32 * (int)(g - (int64_t)y * w.words_per_row);
-            CountT *dst = plane + (int64_t)y * p.pitch + x0;
             uint32_t pairs[16];
             bitcount_pairs(acc[j], pairs);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            for (int i = 0; i < 16; ++i) sh.counts[16 * j + i][tid] = pairs[i];
+        }
+        if (consumers_any(failed)) return;
+        // word f of the tile: pixels 2f and 2f + 1; words past the raster's last
+        // (a partial tile) come from stale bytes and are skipped.  The raster's
+        // width is a whole number of words, so the plane is as dense as it is.
+        constexpr int kPairWords = 16 * kBitsTileWords;
+        const int64_t word0 = (int64_t)tile * kBitsTileWords;
+        const int words = (int)(min((int64_t)kBitsTileWords, w.words - word0) * 16);
+        CountT *dst = plane + word0 * 32;
+        bool under = false;
+        for (int f0 = tid; f0 < kPairWords; f0 += 8 * kBitsConsumers) {
+            uint32_t d[8], old[8][2];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int f = f0 + i * kBitsConsumers;
+                d[i] = 0u;
+                if (f >= words) continue;
+                d[i] = sh.counts[f % (16 * kBitsWordsPerThread)][f / (16 * kBitsWordsPerThread)];
+                if (w.slabs == 1) load_pair(dst + 2 * f, old[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int f = f0 + i * kBitsConsumers;
+                if (f >= words) break;
                 if (w.slabs == 1)
-                    apply_pair_group<CountT>(dst + 16 * h, 16, pairs + 8 * h, sign, flags);
+                    under |= store_pair(dst + 2 * f, old[i], d[i], sign);
                 else
-                    atomic_pair_group<CountT>(dst + 16 * h, pairs + 8 * h, sign, flags);
+                    under |= atomic_pair(dst + 2 * f, d[i], sign);
             }
         }
+        if (under) flag_set(flags, kFlagUnderflow);
+        consumers_sync();   // the next item's counts go to the same words
     }
 }
 
@@ -747,7 +848,7 @@ cudaError_t launch_bits_bulk_t(const BitsWork &w, unsigned grid, const Plane &p,
 cudaError_t launch_count_bits_bulk(const RasterBatch &b, const Plane &p, int sign, int *flags, uint64_t timeout_ns,
                                    const DeviceCaps &caps, cudaStream_t s) {
     if (b.n <= 0 || p.width == 0 || p.height == 0) return cudaSuccess;
-    if (!bits_bulk_compatible(b, p.width, p.height)) return cudaErrorInvalidValue;
+    if (!bits_bulk_compatible(b, p.width, p.height) || p.pitch != p.width) return cudaErrorInvalidValue;
     BitsWork w;
     w.base = static_cast<const uint8_t *>(b.base);
     w.stride = b.member_stride;
