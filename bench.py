@@ -596,7 +596,7 @@ def run_ours(args):
         copy_busy = sum(b - a for a, b in copies)
         n_chunks = sum(1 for k, _, _ in rec if int(k) == 2)
         chunk_used = -(-N // max(1, n_chunks))
-        e2e_launches = 2 if use_direct else n_chunks + 1     # accumulate launches + the render
+        e2e_launches = 3 if use_direct else n_chunks + 2     # the clear, accumulate launches, the render
         e2e = {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": N * P,
                "d2h_bytes_per_step": 5 * P, "ms_per_step": e2e_ms / args.steps,
                "mode": "host_read (kernel loads pinned host memory over the link)" if use_direct
@@ -622,7 +622,7 @@ def run_ours(args):
             cpu_all = cpu_oracle_rate_all_cores(args, args.cpu_seconds)
 
     if rank == 0:
-        launches_per_step = 2
+        launches_per_step = 3   # the clear, the accumulation, the render
         launches_e2e = e2e_launches if e2e else 0
         line = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
