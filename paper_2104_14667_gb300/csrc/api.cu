@@ -39,6 +39,9 @@ thread_local std::string g_begin_error;
 
 enum MemKind { kPageable = 0, kPinned = 1, kDevice = 2, kForeignDevice = 3 };
 constexpr int kDefaultTmaBoxBytes = 256;
+// A context's small device state: the flags, then the histogram scratch.
+constexpr size_t kHistOffset = 256;
+constexpr size_t kStateBytes = kHistOffset + sizeof(cpt::HistScratch);
 enum TraceKind { kTraceUpload = 0, kTraceConvert = 1, kTraceKernel = 2 };
 
 struct Slot {
@@ -76,6 +79,7 @@ struct composite_ctx {
     int array_layers = 0;      // texture path: layers of a slot's array
     Plane plane{};
     int *flags = nullptr;      // device flags
+    cpt::HistScratch *hist_scratch = nullptr;   // after the flags, in one allocation
     int *h_flags = nullptr;    // pinned copy of the flags
     int64_t n_members = 0;
     bool poisoned = false;
@@ -346,7 +350,8 @@ int setup(composite_ctx *ctx) {
     ctx->plane.width = ctx->width;
     ctx->plane.height = ctx->height;
     ctx->plane.count_bits = c.mode == CPT_MODE_COUNT ? c.count_bits : 0;
-    CK(ctx, cudaMalloc(&ctx->flags, cpt::kFlagCount * sizeof(int)));
+    CK(ctx, cudaMalloc(&ctx->flags, kStateBytes));
+    ctx->hist_scratch = reinterpret_cast<cpt::HistScratch *>(reinterpret_cast<uint8_t *>(ctx->flags) + kHistOffset);
     CK(ctx, cudaHostAlloc(&ctx->h_flags, cpt::kFlagCount * sizeof(int), cudaHostAllocDefault));
     memset(ctx->h_flags, 0, cpt::kFlagCount * sizeof(int));
 
@@ -387,7 +392,7 @@ int setup(composite_ctx *ctx) {
     }
     ctx->default_lut = pack_lut(def);
     CK(ctx, cudaMemsetAsync(ctx->plane.data, 0, plane_bytes, ctx->compute));
-    CK(ctx, cudaMemsetAsync(ctx->flags, 0, cpt::kFlagCount * sizeof(int), ctx->compute));
+    CK(ctx, cudaMemsetAsync(ctx->flags, 0, kStateBytes, ctx->compute));
     return CPT_OK;
 }
 
@@ -1077,7 +1082,7 @@ int render(composite_ctx *ctx, void *counts_out, uint8_t *bucket_out, uint8_t *r
     if (out_on_device) {
         cudaError_t e = count ? cpt::launch_render_counts(ctx->plane, n, counts_out, bucket_out,
                                                           reinterpret_cast<uint32_t *>(rgba_out), lut, ctx->caps,
-                                                          ctx->compute, hist_out)
+                                                          ctx->compute, hist_out, ctx->hist_scratch)
                               : cpt::launch_render_mean(ctx->plane, n, mean_out, ctx->caps, ctx->compute);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "render kernel launch");
         return CPT_OK;
@@ -1105,7 +1110,8 @@ int render(composite_ctx *ctx, void *counts_out, uint8_t *bucket_out, uint8_t *r
         cudaError_t e = cpt::launch_render_counts(ctx->plane, n, counts_out ? d_counts : nullptr,
                                                   bucket_out ? d_bucket : nullptr,
                                                   rgba_out ? reinterpret_cast<uint32_t *>(d_rgba) : nullptr,
-                                                  lut, ctx->caps, ctx->compute, hist_out ? d_hist : nullptr);
+                                                  lut, ctx->caps, ctx->compute, hist_out ? d_hist : nullptr,
+                                                  ctx->hist_scratch);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "render kernel launch");
         if (hist_out) CK(ctx, cudaMemcpyAsync(hist_out, d_hist, 256 * sizeof(uint64_t), cudaMemcpyDeviceToHost, ctx->compute));
         if (counts_out) CK(ctx, cudaMemcpyAsync(counts_out, d_counts, (size_t)px * cb, cudaMemcpyDeviceToHost, ctx->compute));

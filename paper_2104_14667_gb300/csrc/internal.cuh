@@ -114,11 +114,18 @@ int encode_tma_map(CUtensorMap *map, const RasterBatch &b, int width, int height
 struct Lut {
     uint32_t rgba[256];
 };
-// hist_out (device, 256 x uint64, may be NULL): zeroed, then the number of
-// pixels in every overlap class, counted in the same pass.
+// Where a histogram render's CTAs add up their classes: device memory of its
+// owner, zero before the first render; renders that share one must not overlap.
+struct HistScratch {
+    unsigned long long bins[256];
+    unsigned int arrived;
+};
+// hist_out (device, 256 x uint64, may be NULL, else with a scratch): the number
+// of pixels in every overlap class, counted in the same pass.
 cudaError_t launch_render_counts(const Plane &p, uint64_t n_members, void *counts_out,
                                  uint8_t *bucket_out, uint32_t *rgba_out, const Lut &lut,
-                                 const DeviceCaps &caps, cudaStream_t s, uint64_t *hist_out = nullptr);
+                                 const DeviceCaps &caps, cudaStream_t s, uint64_t *hist_out = nullptr,
+                                 HistScratch *scratch = nullptr);
 cudaError_t launch_render_mean(const Plane &p, uint64_t n_members, float *mean_out,
                                const DeviceCaps &caps, cudaStream_t s);
 
