@@ -695,12 +695,16 @@ int64_t etimeout(const composite_engine *e) { return e->cfg.wait_timeout_ms > 0 
 
 int ewait(composite_engine *e, cudaEvent_t ev) {
     const auto deadline = std::chrono::steady_clock::now() + std::chrono::milliseconds(etimeout(e));
-    for (cpt::PollPause pause;; pause()) {
+    for (unsigned spin = 0;; ++spin) {
         const cudaError_t r = cudaEventQuery(ev);
         if (r == cudaSuccess) return CPT_OK;
         if (r != cudaErrorNotReady) return ecuda(e, r, "cudaEventQuery");
         if (std::chrono::steady_clock::now() > deadline)
             return efail(e, CPT_ETIMEOUT, "wait exceeded %lld ms", (long long)etimeout(e));
+        if (spin < 200)
+            std::this_thread::yield();
+        else
+            std::this_thread::sleep_for(std::chrono::microseconds(50));
     }
 }
 

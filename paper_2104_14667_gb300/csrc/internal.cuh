@@ -2,9 +2,6 @@
 // Not installed; the public interface is include/composite.h.
 #pragma once
 
-#include <chrono>
-#include <thread>
-
 #include <cuda_runtime.h>
 #include <cuda.h>
 #include <stdint.h>
@@ -149,32 +146,6 @@ bool fault_injected(const char *site);
 // server cycle, engine_chunk_fail=K to staging chunk K of an engine submit's
 // host ops.  Each fails on the host, before that chunk's work is queued.
 int64_t fault_injected_value(const char *site);
-
-// The pause between two polls of a bounded host wait: none for the first
-// polls, about four microseconds for the first two milliseconds, then 50 us of
-// sleep (in fact about 110) -- long waits have time, and tight polling loops
-// were measured to slow copies over the host link.  Eight served sessions took
-// 473 us a pass when the pauses became sleeps after 200 polls, 330 with these.
-class PollPause {
-  public:
-    void operator()() {
-        using namespace std::chrono;
-        if (++polls_ <= 64) {
-            std::this_thread::yield();
-            return;
-        }
-        const auto now = steady_clock::now();
-        if (now - start_ < milliseconds(2)) {
-            while (steady_clock::now() - now < microseconds(4)) std::this_thread::yield();
-        } else {
-            std::this_thread::sleep_for(microseconds(50));
-        }
-    }
-
-  private:
-    std::chrono::steady_clock::time_point start_ = std::chrono::steady_clock::now();
-    unsigned polls_ = 0;
-};
 
 // NVTX range around a host-side phase (a call, a pipeline chunk), for
 // timeline profilers; a no-op call when no profiler is attached.
