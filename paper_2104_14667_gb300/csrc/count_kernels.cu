@@ -40,6 +40,7 @@ count_linear_kernel(RasterBatch b, Plane p, int sign, int *flags, int64_t groups
     const int64_t g = (int64_t)blockIdx.x * kGroups + lane_group;
     uint32_t k[4] = {0u, 0u, 0u, 0u};
     int y = 0, x0 = 0;
+    await_previous();   // every thread: a clear or render before may still be using the plane
     if (g < groups) {
         y = (int)(g / groups_per_row);
         x0 = (int)(g - (int64_t)y * groups_per_row) * 16;
