@@ -604,6 +604,7 @@ struct PlaneRec {
     int64_t n = 0;
     bool alive = false;
     bool poisoned = false;       // a submit failed after its launch may have begun
+    int32_t listed = -1;         // split_ops: the plane's place in the list of the submit's planes
 
     size_t bytes() const { return (size_t)pitch_px * height * (count_bits / 8); }
     int64_t max_members() const { return count_bits == 16 ? 0xFFFFll : 0xFFFFFFFFll; }
@@ -824,7 +825,7 @@ bool plane_ok(const composite_engine *e, int32_t p) {
 // whole served pass 2.88 ms with such items and atomics, 0.47 ms now.  Items
 // of single warps (no slices) took 420 us for the 64 uneven requests' 2.0 GB
 // of masks, items of CTAs take 350 (5.8 TB/s).
-int64_t split_ops(const composite_engine *e, std::vector<OpDesc> *descs) {
+int64_t split_ops(composite_engine *e, std::vector<OpDesc> *descs) {
     const int64_t ctas = (int64_t)e->caps.num_sms * std::min(e->cfg.ctas_per_sm, kResidentCtas);
     const int cfg_slab = e->cfg.slab_members;
     auto slices_of = [](const OpDesc &d, int members) { return !d.bits && members >= kSliceMembers ? kSlices : 1; };
@@ -841,11 +842,21 @@ int64_t split_ops(const composite_engine *e, std::vector<OpDesc> *descs) {
         bool adds = false, removes = false;
         bool chained = false;
     };
-    std::vector<PlaneOps> planes(e->planes.size());
+    // One entry per plane of the submit, not per plane of the engine: tables
+    // over 60000 planes cost a submit of one small op 0.14 ms on the host.
+    std::vector<PlaneOps> planes;
+    for (const OpDesc &d : *descs) e->planes[d.plane_id].listed = -1;
+    for (const OpDesc &d : *descs) {
+        int32_t &at = e->planes[d.plane_id].listed;
+        if (at >= 0) continue;
+        at = (int32_t)planes.size();
+        planes.emplace_back();
+    }
+    auto place = [e](const OpDesc &d) { return (size_t)e->planes[d.plane_id].listed; };
     int64_t steps_once = 0;      // steps of the planes' first ops
     int64_t thread_work = 0;     // (member, group) pairs per thread over all steps
     for (const OpDesc &d : *descs) {
-        PlaneOps &p = planes[d.plane_id];
+        PlaneOps &p = planes[place(d)];
         if (p.ops++ == 0) {
             p.bits = d.bits;
             steps_once += steps_of(d, slices_of(d, d.n));
@@ -868,11 +879,11 @@ int64_t split_ops(const composite_engine *e, std::vector<OpDesc> *descs) {
         order.reserve(descs->size());
         std::vector<std::vector<size_t>> later(planes.size());
         for (size_t i = 0; i < descs->size(); ++i) {
-            const int32_t id = (*descs)[i].plane_id;
+            const size_t id = place((*descs)[i]);
             if (planes[id].chained && planes[id].ops > 1) later[id].push_back(i);
         }
         for (size_t i = 0; i < descs->size(); ++i) {
-            const int32_t id = (*descs)[i].plane_id;
+            const size_t id = place((*descs)[i]);
             if (!(planes[id].chained && planes[id].ops > 1)) {
                 order.push_back((*descs)[i]);
             } else if (later[id].front() == i) {
@@ -885,7 +896,7 @@ int64_t split_ops(const composite_engine *e, std::vector<OpDesc> *descs) {
     int64_t items = 0;
     for (size_t i = 0; i < descs->size();) {
         OpDesc &head = (*descs)[i];
-        const PlaneOps &p = planes[head.plane_id];
+        const PlaneOps &p = planes[place(head)];
         const int chain = p.chained ? p.ops : 1;
         int slab = cfg_slab;
         if (!p.chained && !fills && head.n > kSplitMembers) {
