@@ -22,11 +22,13 @@
 #include <thread>
 #include <vector>
 
+#include <cudaTypedefs.h>
 #include <nvtx3/nvToolsExt.h>
 
 #include "composite.h"
 #include "copy_pool.cuh"
 #include "internal.cuh"
+#include "pinned_range.cuh"
 
 using cpt::DeviceCaps;
 using cpt::Lut;
@@ -510,13 +512,45 @@ bool upload_as_one(const composite_ctx *ctx, const Slot &s, int64_t stride, int6
     return tma_runs(ctx, RasterBatch{s.stage, stride, pitch, c});
 }
 
+// The start and size of the allocation or registration that holds p, as the
+// driver reports them; false where it reports none.
+bool pinned_range(const void *p, uintptr_t *start, size_t *size) {
+    static const PFN_cuPointerGetAttribute_v4000 query = []() -> PFN_cuPointerGetAttribute_v4000 {
+        cudaDriverEntryPointQueryResult q;
+        void *fn = nullptr;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &fn, 4000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            return reinterpret_cast<PFN_cuPointerGetAttribute_v4000>(fn);
+        return nullptr;
+    }();
+    if (!query) return false;
+    const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+    CUdeviceptr first = 0;
+    if (query(&first, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) != CUDA_SUCCESS ||
+        query(size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) != CUDA_SUCCESS)
+        return false;
+    *start = (uintptr_t)first;
+    return true;
+}
+
+// The device mapping of `bytes` bytes of pinned host memory from p, or NULL
+// where p has none or its range ends before they do.
+const void *mapped_range(const void *p, int64_t bytes) {
+    void *mapped = nullptr;
+    if (!cpt::in_one_range(p, bytes, pinned_range)) return nullptr;
+    if (cudaHostGetDevicePointer(&mapped, const_cast<void *>(p), 0) == cudaSuccess) return mapped;
+    cudaGetLastError();
+    return nullptr;
+}
+
 // Uploads c rasters (pinned host or device memory) into a staging buffer laid
 // out with row pitch stage_pitch and raster stride member_bytes: one copy where
 // the layouts agree; pitched copies where pinned rows start on 16-byte
 // boundaries (190-200 GB/s); else a kernel that moves the rows (pinned rasters
 // through their device mapping, over the host link, at 170-180 GB/s), since
 // pitched copies of rows 506 and 3164 bytes apart went at 15 and 58 GB/s, and
-// device rows of 154 floats at 1 TB/s.
+// device rows of 154 floats at 1 TB/s.  Rasters that no one mapped range holds
+// take the pitched copies, which check their ranges themselves.
 int upload(composite_ctx *ctx, uint8_t *dst, const uint8_t *src, int c, int64_t stride,
            int64_t pitch, bool device) {
     const int64_t row = ctx->row_bytes;
@@ -526,12 +560,9 @@ int upload(composite_ctx *ctx, uint8_t *dst, const uint8_t *src, int c, int64_t 
         CK(ctx, cudaMemcpyAsync(dst, src, (size_t)c * ctx->member_bytes, cudaMemcpyDefault, ctx->copy));
         return CPT_OK;
     }
-    void *mapped = nullptr;
+    const void *mapped = nullptr;
     const bool aligned = (reinterpret_cast<uintptr_t>(src) | (uintptr_t)pitch | (uintptr_t)stride) % 16 == 0;
-    if (!device && !aligned && cudaHostGetDevicePointer(&mapped, const_cast<uint8_t *>(src), 0) != cudaSuccess) {
-        cudaGetLastError();
-        mapped = nullptr;
-    }
+    if (!device && !aligned) mapped = mapped_range(src, (c - 1) * stride + (h - 1) * pitch + row);
     if (device || mapped) {
         const RasterBatch b{device ? src : mapped, stride, pitch, c};
         CK(ctx, cpt::launch_repitch(dst, dpitch, ctx->member_bytes, b, row, ctx->height, ctx->copy));
