@@ -1088,6 +1088,13 @@ int composite_remove_members(composite_ctx *ctx, const void *members, int32_t n_
 
 namespace {
 
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return false;
+}
+
 int render(composite_ctx *ctx, void *counts_out, uint8_t *bucket_out, uint8_t *rgba_out, float *mean_out,
            uint64_t *hist_out, int32_t out_on_device, const uint8_t *lut_rgba) {
     const cpt::TraceRange range("composite_render");
@@ -1117,9 +1124,11 @@ int render(composite_ctx *ctx, void *counts_out, uint8_t *bucket_out, uint8_t *r
     const int cb = count ? ctx->cfg.count_bits / 8 : 0;
 
     if (out_on_device) {
+        // a captured render may be replayed beside others of the context
+        cpt::HistScratch *scratch = hist_out && capturing(ctx->compute) ? nullptr : ctx->hist_scratch;
         cudaError_t e = count ? cpt::launch_render_counts(ctx->plane, n, counts_out, bucket_out,
                                                           reinterpret_cast<uint32_t *>(rgba_out), lut, ctx->caps,
-                                                          ctx->compute, hist_out, ctx->hist_scratch)
+                                                          ctx->compute, hist_out, scratch)
                               : cpt::launch_render_mean(ctx->plane, n, mean_out, ctx->caps, ctx->compute);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "render kernel launch");
         return CPT_OK;

@@ -117,8 +117,9 @@ struct HistScratch {
     unsigned long long bins[256];
     unsigned int arrived;
 };
-// hist_out (device, 256 x uint64, may be NULL, else with a scratch): the number
-// of pixels in every overlap class, counted in the same pass.
+// hist_out (device, 256 x uint64, may be NULL): the number of pixels in every
+// overlap class, counted in the same pass; without a scratch into the output,
+// which is cleared first, so that such renders may overlap one another.
 cudaError_t launch_render_counts(const Plane &p, uint64_t n_members, void *counts_out,
                                  uint8_t *bucket_out, uint32_t *rgba_out, const Lut &lut,
                                  const DeviceCaps &caps, cudaStream_t s, uint64_t *hist_out = nullptr,

@@ -23,7 +23,8 @@ constexpr int kCtasPerSm = 16;      // grid cap of the others
 // The totals meet in a scratch that is zero between renders: cleared outputs
 // would need an operation of their own before this one, between kernels that
 // otherwise follow one another closely (509 x 516, two members out and two in:
-// 35.3 us a pass with it, 29.5 without).
+// 35.3 us a pass with it, 29.5 without).  Without a scratch the totals go to
+// the output, cleared by such an operation.
 static_assert(kThreads == 256, "a thread hands over one class");
 template <typename CountT, int kRows, bool kHist, int kUnits>
 __global__ void __launch_bounds__(kThreads, kHist ? kHistCtasPerSm : 1)
@@ -75,7 +76,8 @@ render_counts_kernel(Plane p, ClassDivisor div, CountT *counts_out, uint8_t *buc
     if (kHist) {
         hist_fold(cnt, tot, lane);
         __syncthreads();
-        hist_emit_block(s_hist, kWarps, scratch->bins);
+        hist_emit_block(s_hist, kWarps, scratch ? scratch->bins : hist_out);
+        if (!scratch) return;
         // the last CTA to get here hands the bins over and leaves them zero
         __shared__ int last;
         __threadfence();
@@ -187,6 +189,10 @@ cudaError_t launch_render_counts(const Plane &p, uint64_t n_members, void *count
     const bool u16 = p.count_bits == 16;
     if (hist_out) {
         unsigned long long *h = reinterpret_cast<unsigned long long *>(hist_out);
+        if (!scratch) {
+            const cudaError_t e = cudaMemsetAsync(h, 0, 256 * sizeof(*h), s);
+            if (e != cudaSuccess) return e;
+        }
         return u16 ? render_counts_t<uint16_t, true>(p, n_members, counts_out, bucket_out, rgba_out, lut, h, scratch, caps, s)
                    : render_counts_t<uint32_t, true>(p, n_members, counts_out, bucket_out, rgba_out, lut, h, scratch, caps, s);
     }
