@@ -266,8 +266,13 @@ int composite_load_counts(composite_ctx *ctx, const void *counts, int64_t n_memb
 /* With config.trace = 1: copies up to `capacity` records of 3 floats
  * {kind, start_ms, end_ms} into `records` (host memory), kind 0 = upload,
  * 1 = layout conversion, 2 = accumulation kernel, times relative to the
- * first traced event since the last composite_clear.  Waits (bounded) for
- * the traced work.  *n_out = records available (may exceed capacity). */
+ * first traced event since the last composite_clear.  Uploads and conversions
+ * have a record per chunk, accumulation kernels one per launch.  Masks in
+ * device memory on the texture path are converted several chunks at a time
+ * (CPT_CONVERT_KERNEL): the first of them has the interval of the conversion,
+ * the others empty ones at its end (start_ms = end_ms), so sums and unions of
+ * intervals hold and times per record do not.  Waits (bounded) for the traced
+ * work.  *n_out = records available (may exceed capacity). */
 int composite_trace_read(composite_ctx *ctx, float *records, int32_t capacity, int32_t *n_out);
 
 /* Waits (bounded) for the context's work and frees everything it owns.

@@ -273,7 +273,8 @@ def composite_member_count(ctx) -> int:
 
 
 def composite_trace_read(ctx) -> np.ndarray:
-    """float32[n, 3] records {kind, start_ms, end_ms}."""
+    """float32[n, 3] records {kind, start_ms, end_ms}; chunks that one
+    conversion took together have its interval once, the rest empty ones."""
     lib = load()
     n = ctypes.c_int32()
     _check(lib, ctx, lib.composite_trace_read(ctx, None, 0, ctypes.byref(n)))
