@@ -45,7 +45,7 @@ extern "C" {
 
 typedef struct composite_engine composite_engine;
 
-/* How the accumulate launch hands work items to warps. */
+/* How the accumulate launch hands work items to CTAs. */
 enum {
     CPT_SCHEDULE_PERSISTENT = 0,  /* num_SMs x ctas_per_sm CTAs claim items from a counter */
     CPT_SCHEDULE_GRID = 1         /* one CTA per item; the hardware schedules the CTAs       */

@@ -135,7 +135,8 @@ int composite_server_request_histogram(composite_server *srv, int32_t session, c
 int composite_server_pump(composite_server *srv, int64_t *completed, int32_t capacity, int32_t *n_completed);
 
 /* Pumps until nothing is queued or in flight (bounded by wait_timeout_ms per
- * cycle); completed ids are dropped. */
+ * cycle); completed ids are dropped.  The calling thread polls without sleeping
+ * for two milliseconds after each completion. */
 int composite_server_drain(composite_server *srv);
 
 /* Member count of a session after every queued request (host bookkeeping). */

@@ -12,7 +12,7 @@
 // bound by HBM (large batches) or by its latency (small ones): 4096^2 x 1024
 // takes 2.32 ms, 7.4 TB/s.  Rasters at odd addresses or pitches used to be
 // copied into staging slots first: 1501 x 1103 x 100 with clear and render
-// 338 us, now 61.
+// 338 us, now 46.
 #include <algorithm>
 
 #include "mask_load.cuh"

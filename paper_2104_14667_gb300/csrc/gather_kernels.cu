@@ -7,8 +7,9 @@
 // mapping over the host link, so one launch replaces one copy call per raster
 // (a cycle moves about a thousand).
 //
-// Device rasters at odd pitches or addresses into aligned staging rows, for the
-// paths that need those (tensor maps, float arrays).
+// Rasters at odd pitches or addresses into aligned staging rows: device rasters
+// for the paths that need those (tensor maps, float arrays), pinned host
+// rasters through their device mapping.
 #include <algorithm>
 
 #include "mask_load.cuh"

@@ -67,7 +67,7 @@ cudaError_t launch_gather_rasters(void *dst, const void *src, const int32_t *ids
                                   int64_t raster_bytes, const DeviceCaps &caps, cudaStream_t s);
 // A batch of rasters of `row` bytes by `height` rows, at any alignment, into
 // rows of dpitch and members of dmember bytes (16-byte aligned, zero past the
-// row): device memory only.
+// row) in device memory; b may be the device mapping of pinned host memory.
 cudaError_t launch_repitch(void *dst, int64_t dpitch, int64_t dmember, const RasterBatch &b, int64_t row, int height,
                            cudaStream_t s);
 // Linear rasters (16-byte aligned base, pitch and stride) -> the layers of a

@@ -10,9 +10,10 @@
 // is ordered as ever.
 //
 // A clear, a fold and a render of a small raster are mostly the gaps between
-// them.  Measured, us per pass without and with: 1856 x 2208, four members out
-// and four in with a histogram, 37.0 and 28.7; 1501 x 1103 x 100 53.2 and 45.1;
-// 1024^2 x 16 streamed 104.5 and 100.1; 4096^2 x 1024 2371 and 2361.
+// them.  Measured, us per pass without and with (every kernel waiting): 1856 x
+// 2208, four members out and four in with a histogram, 37.0 and 29.5 to 33.6 by
+// the run; 1501 x 1103 x 100 53.2 and 45.8; 1856 x 2208 x 64 depths 172.4 and
+// 165.6; 1024^2 x 16 streamed 104.3 and 99.2; 4096^2 x 1024 2367 and 2359.
 #pragma once
 
 #include <utility>

@@ -68,8 +68,9 @@ thread_local std::string g_server_error;
 // microseconds for the first two milliseconds, then 50 us of sleep (in fact
 // about 110).  A cycle takes a few hundred microseconds and moves its overflow
 // by a kernel; with sleeps after 200 polls eight sessions took 473 us a pass,
-// 330 with these.  (Waits on the copy engines keep the early sleeps: polling
-// was measured to slow their copies.)
+// 330 with these, for a host core that is busy that long after each completion.
+// (Waits on the copy engines keep the early sleeps: polling was measured to
+// slow their copies.)
 class PollPause {
   public:
     void operator()() {
@@ -599,7 +600,10 @@ int composite_server_begin(composite_server **out, const composite_server_config
         // three persistent CTAs per SM, not all four that fit: the overflow
         // gather kernel on the copy stream then has room beside the engine's
         // launch, and the uploads overlap the folds instead of taking turns
-        // with them (eight sessions of 1024^2 members: 472 against 580 us a pass)
+        // with them (eight sessions of 1024^2 members: 472 against 580 us a pass;
+        // 16 sessions of 4096^2 members at 500 requests/s: bit-packed masks 349
+        // to 355 against 339 to 341 composites/s, byte masks 68 to 69 against
+        // 66 to 69)
         ec.ctas_per_sm = 3;
         ec.upload_stream = s->copy;
         int rc = composite_engine_begin(&s->eng, &ec);

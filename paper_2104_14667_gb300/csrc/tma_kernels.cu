@@ -432,7 +432,6 @@ struct BitsWork {
     const uint8_t *base;
     int64_t stride;          // member stride, bytes
     int64_t words;           // 32-pixel words per member
-    int words_per_row;
     int tiles;
     int slabs;
     int slab_stages;
@@ -852,8 +851,7 @@ cudaError_t launch_count_bits_bulk(const RasterBatch &b, const Plane &p, int sig
     BitsWork w;
     w.base = static_cast<const uint8_t *>(b.base);
     w.stride = b.member_stride;
-    w.words_per_row = p.width / 32;
-    w.words = (int64_t)w.words_per_row * p.height;
+    w.words = (int64_t)(p.width / 32) * p.height;
     const int64_t tiles = (w.words + kBitsTileWords - 1) / kBitsTileWords;
     if (tiles > (1 << 24)) return cudaErrorInvalidValue;
     w.tiles = (int)tiles;

@@ -26,7 +26,7 @@ import os
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 # the sources the linear count kernel is built from
-KERNEL_SOURCES = ("count_kernels.cu", "mask_load.cuh", "device_common.cuh")
+KERNEL_SOURCES = ("count_kernels.cu", "mask_load.cuh", "overlap.cuh", "device_common.cuh")
 
 
 def kernel_source_hash() -> str:
