@@ -42,6 +42,10 @@ struct alignas(128) TmaShared {
     uint8_t stage[kStages][kBoxBytes];
     uint64_t full[kStages];
     uint64_t empty[kStages];
+    // runs into padded planes: a warp's counts (or sums) on their way to the
+    // lanes that update them, 16 per thread and a pad that keeps both orders
+    // off shared banks
+    uint32_t counts[kConsumers / 32][32 * 17];
     int abort;
 };
 constexpr size_t kSmemBytes = sizeof(TmaShared) + 128;   // + alignment slack
@@ -160,36 +164,64 @@ __device__ void produce(TmaShared &sh, const CUtensorMap *map, int tiles, int ti
 // unaligned widths 2 to 15 times faster than by way of staging slots.
 constexpr int kRunBytes = kMemberPlaneBytes;
 constexpr int kRunElem = 8;
+constexpr int kPaddedRuns = -1;   // kBoxX of the kernels below
 
-// 16 counts of pixels i .. i + valid - 1 (in the run's order) folded into a
-// plane whose rows are padded: pixel by pixel, on into the next row.
+// Runs into planes whose rows are padded.  A thread holds the counts (or sums)
+// of consecutive pixels, which from there take an access of a sector for every
+// lane of a warp and pixel.  They change hands through shared memory instead:
+// lane l of a warp updates pixels first + l + 32 j of the warp's part of the
+// run.  Where those lie needs no member, so that their old values are on their
+// way while the warp waits for the first box.  Measured, us with clear and
+// render, updated from the threads that hold them / this way: 4090 x 2048 x 1
+// masks 147 / 80, x 16 167 / 83, 8191 x 4096 x 1 depths 728 / 473.
+
+// Where pixels first + lane + 32 j lie, NULL from the `left`th of the warp's on.
+template <typename T, int kCount>
+__device__ __forceinline__ void run_places(T *plane, int64_t pitch, int width, int64_t first, int64_t left, T *(&at)[kCount]) {
+    const int lane = threadIdx.x & 31;
+    int64_t y = (first + lane) / width;
+    int x = (int)(first + lane - y * width);
+    const int dy = 32 / width, dx = 32 % width;
+#pragma unroll
+    for (int j = 0; j < kCount; ++j) {
+        at[j] = lane + 32 * j < left ? plane + y * pitch + x : nullptr;
+        y += dy;
+        x += dx;
+        if (x >= width) {
+            x -= width;
+            ++y;
+        }
+    }
+}
+
+// The warp's counts (16 to a lane in `wide`) folded into the places `at` with
+// the values `old`.  The whole warp calls.
 template <typename CountT>
-__device__ __forceinline__ void apply_count_run(CountT *plane, int64_t pitch, int width, int64_t i, int valid,
-                                                const uint32_t (&wide)[16], int sign, int *flags) {
-    const int64_t y = i / width;
-    int x = (int)(i - y * width);
-    CountT *row = plane + y * pitch;
+__device__ __forceinline__ void apply_count_run(CountT *const (&at)[16], const uint32_t (&old)[16], const uint32_t (&wide)[16],
+                                                uint32_t *part, int sign, int *flags) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) part[17 * lane + j] = wide[j];
+    __syncwarp();
     bool under = false;
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
-        if (j >= valid) break;
-        const uint32_t old = row[x];
-        under |= sign < 0 && wide[j] > old;
-        row[x] = (CountT)(sign > 0 ? old + wide[j] : old - wide[j]);
-        if (++x == width) {
-            x = 0;
-            row += pitch;
-        }
+        if (!at[j]) continue;
+        const int q = lane + 32 * j;
+        const uint32_t d = part[17 * (q / 16) + q % 16];
+        under |= sign < 0 && d > old[j];
+        *at[j] = (CountT)(sign > 0 ? old[j] + d : old[j] - d);
     }
     if (under) flag_set(flags, kFlagUnderflow);
+    __syncwarp();   // the next tile's counts go to the same words
 }
 
-// kBoxX = 0: runs.
+// kBoxX = 0: runs; kPaddedRuns: runs into a plane of padded rows.
 template <typename CountT, int kBoxX>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 count_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members, int sign,
                  int *flags, uint64_t timeout_ns) {
-    constexpr bool kRun = kBoxX == 0;
+    constexpr bool kRun = kBoxX <= 0, kPadded = kBoxX == kPaddedRuns;
     constexpr int kWidth = kRun ? kRunBytes : kBoxX;
     constexpr int kRows = kMemberPlaneBytes / kWidth;
     constexpr int kGroupsPerRow = kWidth / 16;
@@ -228,12 +260,20 @@ count_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members
         for (int j = 0; j < 16; ++j) wide[j] = 0;
         uint32_t k0 = 0, k1 = 0, k2 = 0, k3 = 0;
         int packed_members = 0;
+        CountT *at[16];
+        uint32_t old[16];
+        if constexpr (kPadded) {
+            const int64_t first = (int64_t)tile * kRunBytes + offset / 512 * 512;   // the warp's
+            run_places(plane, p.pitch, p.width, first, pixels - first, at);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) old[j] = at[j] ? (uint32_t)*at[j] : 0u;
+        }
         for (int slab = 0; slab < slabs; ++slab, ++it) {
             const int s = it % kStages;
-            if (!wait_bounded(&sh.full[s], (it / kStages) & 1u, timeout_ns, &sh.abort)) {
+            if (!__all_sync(0xFFFFFFFFu, wait_bounded(&sh.full[s], (it / kStages) & 1u, timeout_ns, &sh.abort))) {
                 flag_set(flags, kFlagTimeout);
                 sh.abort = 1;
-                return;
+                return;   // the whole warp
             }
             const uint8_t *box = sh.stage[s] + offset;
 #pragma unroll
@@ -255,12 +295,10 @@ count_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members
         widen16(wide, k0, k1, k2, k3);
         if constexpr (kRun) {
             const int64_t i = (int64_t)tile * kRunBytes + offset;
-            const int valid = (int)min((int64_t)16, pixels - i);
-            if (valid <= 0) continue;
-            if (p.pitch == p.width)
+            if constexpr (kPadded)
+                apply_count_run<CountT>(at, old, wide, sh.counts[threadIdx.x / 32], sign, flags);
+            else if (i < pixels)
                 apply_count_group<CountT>(plane + i, 16, wide, sign, flags);
-            else
-                apply_count_run<CountT>(plane, p.pitch, p.width, i, valid, wide, sign, flags);
             continue;
         }
         const int y = ty * kRows + row;
@@ -275,7 +313,7 @@ template <int kBoxX>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 depth_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members, int sign,
                  int *flags, uint64_t timeout_ns) {
-    constexpr bool kRun = kBoxX == 0;
+    constexpr bool kRun = kBoxX <= 0, kPadded = kBoxX == kPaddedRuns;
     constexpr int kWidth = kRun ? kRunBytes : kBoxX;
     constexpr int kRows = kMemberPlaneBytes / kWidth;
     constexpr int kGroupsPerRow = kWidth / 16;
@@ -312,12 +350,19 @@ depth_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         const int tx = tile % tiles_x, ty = tile / tiles_x;
         float acc[4] = {0.f, 0.f, 0.f, 0.f}, block[4] = {0.f, 0.f, 0.f, 0.f};
+        float *at[4], old[4];
+        if constexpr (kPadded) {
+            const int64_t first = (int64_t)tile * kBoxXElems + grp / 32 * 128;   // the warp's
+            run_places(plane, p.pitch, p.width, first, pixels - first, at);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) old[j] = at[j] ? *at[j] : 0.f;
+        }
         for (int slab = 0; slab < slabs; ++slab, ++it) {
             const int s = it % kStages;
-            if (!wait_bounded(&sh.full[s], (it / kStages) & 1u, timeout_ns, &sh.abort)) {
+            if (!__all_sync(0xFFFFFFFFu, wait_bounded(&sh.full[s], (it / kStages) & 1u, timeout_ns, &sh.abort))) {
                 flag_set(flags, kFlagTimeout);
                 sh.abort = 1;
-                return;
+                return;   // the whole warp
             }
             const uint8_t *box = sh.stage[s] + offset;
             // eight members a tree, 64 a block, then the total: as the linear path
@@ -342,23 +387,17 @@ depth_tma_kernel(const __grid_constant__ CUtensorMap map, Plane p, int n_members
         }
         if constexpr (kRun) {
             const int64_t i = (int64_t)tile * kBoxXElems + grp * 4;
-            const int valid = (int)min((int64_t)4, pixels - i);
-            if (valid <= 0) continue;
-            if (p.pitch == p.width) {
-                apply_depth_group(plane + i, 4, acc, sign);
-            } else {
-                int64_t py = i / p.width;
-                int px = (int)(i - py * p.width);
+            if constexpr (kPadded) {
+                float *part = reinterpret_cast<float *>(sh.counts[threadIdx.x / 32]);
+                const int lane = threadIdx.x & 31;
+                *reinterpret_cast<float4 *>(part + 4 * lane) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+                __syncwarp();
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (j >= valid) break;
-                    float *dst = plane + py * p.pitch + px;
-                    *dst = sign > 0 ? *dst + acc[j] : *dst - acc[j];
-                    if (++px == p.width) {
-                        px = 0;
-                        ++py;
-                    }
-                }
+                for (int j = 0; j < 4; ++j)
+                    if (at[j]) *at[j] = sign > 0 ? old[j] + part[lane + 32 * j] : old[j] - part[lane + 32 * j];
+                __syncwarp();   // the next tile's sums go to the same words
+            } else if (i < pixels) {
+                apply_depth_group(plane + i, 4, acc, sign);
             }
             continue;
         }
@@ -725,9 +764,9 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encoder() {
     return fn;
 }
 
-// Tiles of a plane for boxes of box_bytes by rows, or runs (box_bytes 0).
+// Tiles of a plane for boxes of box_bytes by rows, or runs (box_bytes 0 or less).
 int tma_tiles(const Plane &p, int elem_bytes, int box_bytes) {
-    if (box_bytes == 0) return (int)(((int64_t)p.width * p.height * elem_bytes + kRunBytes - 1) / kRunBytes);
+    if (box_bytes <= 0) return (int)(((int64_t)p.width * p.height * elem_bytes + kRunBytes - 1) / kRunBytes);
     const int box_px = box_bytes / elem_bytes, rows = kMemberPlaneBytes / box_bytes;
     return ((p.width + box_px - 1) / box_px) * ((p.height + rows - 1) / rows);
 }
@@ -814,6 +853,9 @@ cudaError_t launch_count_tma(const CUtensorMap &map, const RasterBatch &b, const
     const bool u16 = p.count_bits == 16;
     switch (box_bytes) {
         case kTmaRuns:
+            if (p.pitch != p.width)
+                return u16 ? launch_count_tma_t<uint16_t, kPaddedRuns>(map, b, p, sign, flags, timeout_ns, caps, s)
+                           : launch_count_tma_t<uint32_t, kPaddedRuns>(map, b, p, sign, flags, timeout_ns, caps, s);
             return u16 ? launch_count_tma_t<uint16_t, 0>(map, b, p, sign, flags, timeout_ns, caps, s)
                        : launch_count_tma_t<uint32_t, 0>(map, b, p, sign, flags, timeout_ns, caps, s);
         case 64:
@@ -876,7 +918,9 @@ cudaError_t launch_depth_tma(const CUtensorMap &map, const RasterBatch &b, const
                              cudaStream_t s) {
     if (b.n <= 0) return cudaSuccess;
     switch (box_bytes) {
-        case kTmaRuns: return launch_depth_tma_t<0>(map, b, p, sign, flags, timeout_ns, caps, s);
+        case kTmaRuns:
+            return p.pitch != p.width ? launch_depth_tma_t<kPaddedRuns>(map, b, p, sign, flags, timeout_ns, caps, s)
+                                      : launch_depth_tma_t<0>(map, b, p, sign, flags, timeout_ns, caps, s);
         case 64: return launch_depth_tma_t<64>(map, b, p, sign, flags, timeout_ns, caps, s);
         case 128: return launch_depth_tma_t<128>(map, b, p, sign, flags, timeout_ns, caps, s);
         case 256: return launch_depth_tma_t<256>(map, b, p, sign, flags, timeout_ns, caps, s);
