@@ -565,7 +565,8 @@ int upload(composite_ctx *ctx, uint8_t *dst, const uint8_t *src, int c, int64_t 
     if (!device && !aligned) mapped = mapped_range(src, (c - 1) * stride + (h - 1) * pitch + row);
     if (device || mapped) {
         const RasterBatch b{device ? src : mapped, stride, pitch, c};
-        CK(ctx, cpt::launch_repitch(dst, dpitch, ctx->member_bytes, b, row, ctx->height, ctx->copy));
+        const bool leave_room = !device && ctx->cfg.read_path == CPT_READ_TMA;
+        CK(ctx, cpt::launch_repitch(dst, dpitch, ctx->member_bytes, b, row, ctx->height, leave_room, ctx->caps, ctx->copy));
     } else if (stride == pitch * h) {
         CK(ctx, cudaMemcpy2DAsync(dst, dpitch, src, pitch, row, (size_t)c * h, cudaMemcpyDefault, ctx->copy));
     } else {

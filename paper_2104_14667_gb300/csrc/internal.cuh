@@ -68,8 +68,9 @@ cudaError_t launch_gather_rasters(void *dst, const void *src, const int32_t *ids
 // A batch of rasters of `row` bytes by `height` rows, at any alignment, into
 // rows of dpitch and members of dmember bytes (16-byte aligned, zero past the
 // row) in device memory; b may be the device mapping of pinned host memory.
+// leave_room: a TMA kernel finds room to run beside this one.
 cudaError_t launch_repitch(void *dst, int64_t dpitch, int64_t dmember, const RasterBatch &b, int64_t row, int height,
-                           cudaStream_t s);
+                           bool leave_room, const DeviceCaps &caps, cudaStream_t s);
 // Linear rasters (16-byte aligned base, pitch and stride) -> the layers of a
 // cudaArray of 16-byte texels, through a surface object.
 cudaError_t launch_convert_to_array(const void *src, int64_t pitch, int64_t member_stride,
