@@ -546,11 +546,17 @@ const void *mapped_range(const void *p, int64_t bytes) {
 // Uploads c rasters (pinned host or device memory) into a staging buffer laid
 // out with row pitch stage_pitch and raster stride member_bytes: one copy where
 // the layouts agree; pitched copies where pinned rows start on 16-byte
-// boundaries (190-200 GB/s); else a kernel that moves the rows (pinned rasters
-// through their device mapping, over the host link, at 170-180 GB/s), since
-// pitched copies of rows 506 and 3164 bytes apart went at 15 and 58 GB/s, and
-// device rows of 154 floats at 1 TB/s.  Rasters that no one mapped range holds
-// take the pitched copies, which check their ranges themselves.
+// boundaries (190-200 GB/s) or are long; else a kernel that moves the rows
+// (pinned rasters through their device mapping, over the host link, at 170-190
+// GB/s), since pitched copies of rows 506 and 3164 bytes apart went at 15 and
+// 58 GB/s, and device rows of 154 floats at 1 TB/s.  Rasters that no one mapped
+// range holds take the pitched copies, which check their ranges themselves.
+// Pitched copies gain with the row's length (GB/s, 16 rasters of 1500 rows off
+// 16-byte boundaries, copies / kernel): 4000 bytes 70 / 185, 8000 116 / 190,
+// 12000 151 / 185, 16000 166 / 184, 17600 171 / 184, 18000 175 / 174, 19200 186 /
+// 182, 20000 194 / 173, 24000 201 / 172, 32752 187 / 176.
+constexpr int64_t kLongRowBytes = 19000;
+
 int upload(composite_ctx *ctx, uint8_t *dst, const uint8_t *src, int c, int64_t stride,
            int64_t pitch, bool device) {
     const int64_t row = ctx->row_bytes;
@@ -562,7 +568,7 @@ int upload(composite_ctx *ctx, uint8_t *dst, const uint8_t *src, int c, int64_t 
     }
     const void *mapped = nullptr;
     const bool aligned = (reinterpret_cast<uintptr_t>(src) | (uintptr_t)pitch | (uintptr_t)stride) % 16 == 0;
-    if (!device && !aligned) mapped = mapped_range(src, (c - 1) * stride + (h - 1) * pitch + row);
+    if (!device && !aligned && row < kLongRowBytes) mapped = mapped_range(src, (c - 1) * stride + (h - 1) * pitch + row);
     if (device || mapped) {
         const RasterBatch b{device ? src : mapped, stride, pitch, c};
         const bool leave_room = !device && ctx->cfg.read_path == CPT_READ_TMA;

@@ -1,8 +1,13 @@
-"""Pinned rows off 16-byte boundaries on their way through the staging slots: the
+"""Pinned rows off 16-byte boundaries on their way through the staging slots:
+rows on both sides of the length from which pitched copies move them, and the
 fold of a chunk beside the upload of the next."""
 import time
 
+import numpy as np
 import pytest
+
+import oracle
+import synth
 
 torch = pytest.importorskip("torch")
 from paper_2104_14667_gb300 import binding  # noqa: E402
@@ -15,6 +20,30 @@ def pinned(n, h, w, pad, gap, dtype):
     stride = pitch * h + gap
     buf = torch.ones((n - 1) * stride + (h - 1) * pitch + w, dtype=dtype).pin_memory()
     return buf.as_strided((n, h, w), (stride, pitch, 1))
+
+
+@pytest.mark.parametrize("path", ["linear", "texture", "tma"])
+@pytest.mark.parametrize("w", [18983, 18984, 18999, 19000, 19001])
+def test_rows_around_the_length(w, path):
+    n, h = 5, 6
+    m = synth.random_masks(w, n, h, w)
+    src = pinned(n, h, w, 3, 7, torch.uint8)
+    src.copy_(torch.from_numpy(m))
+    with binding.Composite(w, h, read_path=path, chunk_members=2) as comp:
+        comp.add(src)
+        comp.remove(src[:1])
+        np.testing.assert_array_equal(comp.render_host()["counts"].astype(np.int64), oracle.count(m[1:]))
+
+
+@pytest.mark.parametrize("path", ["linear", "texture", "tma"])
+def test_long_rows_of_depths(path):
+    n, h, w = 4, 5, 5003   # rows of 20012 bytes
+    d = np.random.default_rng(3).integers(0, 64, (n, h, w)).astype(np.float32)   # sums exact in any order
+    src = pinned(n, h, w, 1, 1, torch.float32)
+    src.copy_(torch.from_numpy(d))
+    with binding.Composite(w, h, read_path=path, mode="mean_depth", chunk_members=1) as comp:
+        comp.add(src)
+        np.testing.assert_array_equal(comp.render_host()["mean"], d.sum(axis=0) / np.float32(n))
 
 
 def pass_seconds(w, h, src, path) -> float:
@@ -43,3 +72,12 @@ def test_a_fold_runs_beside_the_next_upload():
     # both wait for the link, 2.86 ms the first; 4.1 in every other context where
     # folds found no room beside the next upload and took turns with it
     assert max(took) < 1.25 * copies, (took, copies)
+
+
+def test_long_rows_take_no_longer_than_aligned_ones():
+    n, h, w = 16, 1500, 6001
+    odd = pinned(n, h, w, 1, 5, torch.float32)
+    even = pinned(n, h, w, 3, 0, torch.float32)      # rows on 16-byte boundaries: pitched copies
+    took = [pass_seconds(w, h, src, "linear") for src in (odd, even)]
+    # 2.86 ms both; 3.35 the first when a kernel moved rows of any length
+    assert took[0] < 1.07 * took[1], took
