@@ -727,22 +727,17 @@ Lut make_lut(const uint8_t *rgba) {
 // Bytes ahead of a submit's op descriptors: the item counter, zero.
 constexpr size_t kCounterBytes = 16;
 
-// Op descriptors as a submit uploads them.
-std::vector<unsigned char> op_blob(const std::vector<OpDesc> &descs) {
-    std::vector<unsigned char> blob(kCounterBytes + descs.size() * sizeof(OpDesc), 0);
-    if (!descs.empty()) memcpy(blob.data() + kCounterBytes, descs.data(), descs.size() * sizeof(OpDesc));
-    return blob;
-}
-
 // Copies `bytes` of descriptors into the next slot of the upload ring
 // and queues their upload, on the upload stream when the engine has one (so
 // that small uploads follow the caller's own uploads in order instead of
-// waiting behind them on a copy engine); returns the slot.  The caller
-// records slot->consumed on the engine stream after the launch that reads it.
+// waiting behind them on a copy engine); returns the slot.  `head` zero bytes
+// come first.  The caller records slot->consumed on the engine stream after the
+// launch that reads it.
 int upload(composite_engine *e, Upload *ring, int *idx, const void *src, size_t bytes, Upload **slot,
-           cudaStream_t on = nullptr) {
+           cudaStream_t on = nullptr, size_t head = 0) {
     Upload &u = ring[*idx];
     *idx = (*idx + 1) % kUploadRing;
+    bytes += head;
     if (u.used) {
         int rc = ewait(e, u.done);
         if (rc) return rc;
@@ -758,7 +753,8 @@ int upload(composite_engine *e, Upload *ring, int *idx, const void *src, size_t 
         ECK(e, cudaHostAlloc(&u.h, cap, cudaHostAllocDefault));
         u.cap = cap;
     }
-    memcpy(u.h, src, bytes);
+    if (head) memset(u.h, 0, head);
+    memcpy(static_cast<unsigned char *>(u.h) + head, src, bytes - head);
     if (us != e->stream && u.used) ECK(e, cudaStreamWaitEvent(us, u.consumed, 0));
     ECK(e, cudaMemcpyAsync(u.d, u.h, bytes, cudaMemcpyHostToDevice, us));
     ECK(e, cudaEventRecord(u.done, us));
@@ -841,22 +837,27 @@ int64_t split_ops(composite_engine *e, std::vector<OpDesc> *descs) {
         bool single = true;     // every op is one slab
         bool adds = false, removes = false;
         bool chained = false;
+        bool together = true;   // its ops follow one another in the list
+        size_t last = 0;        // its last op in the list
     };
     // One entry per plane of the submit, not per plane of the engine: tables
     // over 60000 planes cost a submit of one small op 0.14 ms on the host.
     std::vector<PlaneOps> planes;
+    planes.reserve(descs->size());
     for (const OpDesc &d : *descs) e->planes[d.plane_id].listed = -1;
-    for (const OpDesc &d : *descs) {
-        int32_t &at = e->planes[d.plane_id].listed;
-        if (at >= 0) continue;
-        at = (int32_t)planes.size();
-        planes.emplace_back();
-    }
     auto place = [e](const OpDesc &d) { return (size_t)e->planes[d.plane_id].listed; };
     int64_t steps_once = 0;      // steps of the planes' first ops
     int64_t thread_work = 0;     // (member, group) pairs per thread over all steps
-    for (const OpDesc &d : *descs) {
-        PlaneOps &p = planes[place(d)];
+    for (size_t i = 0; i < descs->size(); ++i) {
+        const OpDesc &d = (*descs)[i];
+        int32_t &listed = e->planes[d.plane_id].listed;
+        if (listed < 0) {
+            listed = (int32_t)planes.size();
+            planes.emplace_back();
+        }
+        PlaneOps &p = planes[listed];
+        p.together = p.together && (p.ops == 0 || p.last + 1 == i);
+        p.last = i;
         if (p.ops++ == 0) {
             p.bits = d.bits;
             steps_once += steps_of(d, slices_of(d, d.n));
@@ -874,21 +875,28 @@ int64_t split_ops(composite_engine *e, std::vector<OpDesc> *descs) {
         p.chained = p.ops > 0 && p.single && p.bits >= 0 && p.members <= std::max(cfg_slab, e->cfg.item_member_groups) &&
                     (fills || p.members <= kSplitMembers || (p.adds && p.removes));
     // a plane's chained ops one after another, at the place of its first
-    {
+    bool in_order = true;
+    for (const PlaneOps &p : planes) in_order = in_order && (p.together || !p.chained);
+    if (!in_order) {
+        constexpr size_t kNone = ~(size_t)0;
+        std::vector<size_t> next(descs->size(), kNone);   // the op's successor in its chain
+        std::vector<size_t> first(planes.size(), kNone), last(planes.size(), kNone);
+        for (size_t i = 0; i < descs->size(); ++i) {
+            const size_t at = place((*descs)[i]);
+            if (first[at] == kNone)
+                first[at] = i;
+            else
+                next[last[at]] = i;
+            last[at] = i;
+        }
         std::vector<OpDesc> order;
         order.reserve(descs->size());
-        std::vector<std::vector<size_t>> later(planes.size());
         for (size_t i = 0; i < descs->size(); ++i) {
-            const size_t id = place((*descs)[i]);
-            if (planes[id].chained && planes[id].ops > 1) later[id].push_back(i);
-        }
-        for (size_t i = 0; i < descs->size(); ++i) {
-            const size_t id = place((*descs)[i]);
-            if (!(planes[id].chained && planes[id].ops > 1)) {
+            const size_t at = place((*descs)[i]);
+            if (!planes[at].chained)
                 order.push_back((*descs)[i]);
-            } else if (later[id].front() == i) {
-                for (size_t j : later[id]) order.push_back((*descs)[j]);
-            }
+            else if (first[at] == i)
+                for (size_t j = i; j != kNone; j = next[j]) order.push_back((*descs)[j]);
         }
         descs->swap(order);
     }
@@ -1233,8 +1241,7 @@ int launch_ops(composite_engine *e, const composite_op *ops, int32_t n_ops, bool
     int rc = plan_ops(e, ops, n_ops, &descs, &items, &n_after, false, false);
     if (rc || items == 0) return rc;
     Upload *u = nullptr;
-    const std::vector<unsigned char> blob = op_blob(descs);
-    rc = upload(e, e->up_ops, &e->up_i, blob.data(), blob.size(), &u, desc_stream);
+    rc = upload(e, e->up_ops, &e->up_i, descs.data(), descs.size() * sizeof(OpDesc), &u, desc_stream, kCounterBytes);
     if (rc) return rc;
     if (cpt::fault_injected("engine_submit")) return efail(e, CPT_ECUDA, "submit refused before its launch (injected)");
     *launched = true;   // from here on the launch may have begun
@@ -1353,8 +1360,7 @@ int submit_internal(composite_engine *e, const composite_op *ops, int32_t n_ops)
     if (host_ops.empty()) {
         if (items > 0) {
             Upload *u = nullptr;
-            const std::vector<unsigned char> blob = op_blob(descs);
-            rc = upload(e, e->up_ops, &e->up_i, blob.data(), blob.size(), &u);
+            rc = upload(e, e->up_ops, &e->up_i, descs.data(), descs.size() * sizeof(OpDesc), &u, nullptr, kCounterBytes);
             if (rc) return rc;   // nothing launched: every plane is as before
             if (cpt::fault_injected("engine_submit"))
                 return efail(e, CPT_ECUDA, "submit refused before its launch (injected)");
