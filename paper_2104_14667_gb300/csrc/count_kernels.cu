@@ -273,6 +273,10 @@ cudaError_t launch_depth_t(const RasterBatch &b, const Plane &p, int sign, const
     return cudaGetLastError();
 }
 
+// From this size on two memsets are quicker than the kernel (134 MB 22.7 us
+// either way, 196 MB 30.4 and 31.8, 268 MB 39.8 and 42.3).
+constexpr int64_t kMemsetBytes = 144ll << 20;
+
 // Counts (or sums) and device flags to zero, in one launch.
 __global__ void __launch_bounds__(kThreads)
 clear_plane_kernel(uint4 *data, int64_t words, int *flags) {
@@ -285,6 +289,10 @@ clear_plane_kernel(uint4 *data, int64_t words, int *flags) {
 }  // namespace
 
 cudaError_t launch_clear_plane(void *data, int64_t bytes, int *flags, const DeviceCaps &caps, cudaStream_t s) {
+    if (bytes >= kMemsetBytes) {
+        const cudaError_t e = cudaMemsetAsync(flags, 0, kFlagCount * sizeof(int), s);
+        return e != cudaSuccess ? e : cudaMemsetAsync(data, 0, (size_t)bytes, s);
+    }
     const int64_t words = bytes / 16;   // plane rows are whole 16-byte vectors
     const int64_t blocks = std::min<int64_t>((words + 4 * kThreads - 1) / (4 * kThreads), 8ll * caps.num_sms);
     launch_overlapped(clear_plane_kernel, (unsigned)std::max<int64_t>(1, blocks), kThreads, 0, s, static_cast<uint4 *>(data), words, flags);
