@@ -56,7 +56,9 @@ typedef struct composite_engine_config {
                                  default stream (ordered with the caller's work there) */
     int32_t slab_members;     /* most members of an op per work item, 1..255; 0 = 128  */
     int32_t ctas_per_sm;      /* persistent CTAs of 256 threads per SM, 1..8; 0 = 5;
-                                 more than four run as four, all that fit             */
+                                 more than four run as four, all that fit (or as five
+                                 where bit-packed ops of several slabs are most of a
+                                 submit's work)                                       */
     int64_t wait_timeout_ms;  /* bound on host waits; 0 = 10000                        */
     int32_t schedule;         /* CPT_SCHEDULE_*; default CPT_SCHEDULE_PERSISTENT       */
     void *upload_stream;      /* cudaStream_t for the engine's small host-to-device

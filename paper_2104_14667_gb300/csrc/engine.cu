@@ -42,6 +42,12 @@ constexpr int kSplitMembers = 32;      // shortest slab that a launch short of i
 constexpr int kSlices = 4;             // slices of a CTA's threads on items of kSliceMembers members or more
 constexpr int kSliceMembers = 32;
 constexpr int kResidentCtas = 4;       // CTAs per SM that the accumulate kernels' registers allow
+// A launch of bit-packed ops that are mostly of several slabs, whose counts go
+// into the plane by atomics, waits for those: five CTAs per SM (on 48 registers)
+// hide more of them.  us, four / five: one plane of 4000 x 3000 x 600, 16-bit
+// counts 708 / 584, 32-bit 728 / 606; single slabs are better off with four:
+// eight planes of 1024^2 x 128, 32-bit 90 / 125.
+constexpr int kDeepBitsCtas = 5;
 
 struct OpDesc {
     const uint8_t *base;
@@ -393,8 +399,8 @@ __device__ __forceinline__ void run_item(const OpDesc *head, uint32_t item, Item
 // At most four CTAs per SM are resident, on 64 registers: five on 48 spilled
 // and were slower (64 uneven requests with clear and render: 421 against 400
 // us).  Two or three of them leave room for a kernel on another stream.
-template <int kFormats>
-__global__ void __launch_bounds__(kThreads, kResidentCtas)
+template <int kFormats, int kCtas>
+__global__ void __launch_bounds__(kThreads, kCtas)
 engine_accumulate_kernel(const OpDesc *ops, int n_ops, uint32_t n_items, uint32_t *counter, int *flags) {
     __shared__ ItemShared sh;
     __shared__ uint32_t s_starts[kSmemStarts];
@@ -414,8 +420,8 @@ engine_accumulate_kernel(const OpDesc *ops, int n_ops, uint32_t n_items, uint32_
 }
 
 // Grid schedule: a CTA per item; the hardware block scheduler balances them.
-template <int kFormats>
-__global__ void __launch_bounds__(kThreads, kResidentCtas)
+template <int kFormats, int kCtas>
+__global__ void __launch_bounds__(kThreads, kCtas)
 engine_accumulate_grid_kernel(const OpDesc *ops, int n_ops, int *flags) {
     __shared__ ItemShared sh;
     const uint32_t item = blockIdx.x;
@@ -1043,30 +1049,38 @@ int plan_render(composite_engine *e, const composite_render_op *ops, int32_t n_o
     return CPT_OK;
 }
 
-unsigned persistent_grid(const composite_engine *e, int64_t items) {
-    const int64_t cap = (int64_t)e->caps.num_sms * std::min(e->cfg.ctas_per_sm, kResidentCtas);
+unsigned persistent_grid(const composite_engine *e, int64_t items, int resident) {
+    const int64_t cap = (int64_t)e->caps.num_sms * std::min(e->cfg.ctas_per_sm, resident);
     return (unsigned)std::max<int64_t>(1, std::min(cap, items));
 }
 
-template <int kFormats>
+template <int kFormats, int kCtas = kResidentCtas>
 void launch_accumulate_t(composite_engine *e, const OpDesc *ops, int n_ops, int64_t n_items, uint32_t *counter) {
-    const unsigned grid = persistent_grid(e, n_items);
+    const unsigned grid = persistent_grid(e, n_items, kCtas);
     const uint32_t items = (uint32_t)n_items;
     if (e->cfg.schedule == CPT_SCHEDULE_GRID)
-        engine_accumulate_grid_kernel<kFormats><<<items, kThreads, 0, e->stream>>>(ops, n_ops, e->d_flags);
+        engine_accumulate_grid_kernel<kFormats, kCtas><<<items, kThreads, 0, e->stream>>>(ops, n_ops, e->d_flags);
     else
-        engine_accumulate_kernel<kFormats><<<grid, kThreads, 0, e->stream>>>(ops, n_ops, items, counter, e->d_flags);
+        engine_accumulate_kernel<kFormats, kCtas><<<grid, kThreads, 0, e->stream>>>(ops, n_ops, items, counter, e->d_flags);
 }
 
 // counter: a zeroed device word (persistent schedule).
 int launch_accumulate(composite_engine *e, const void *d_ops, const std::vector<OpDesc> &descs, int64_t n_items,
                       uint32_t *counter) {
     bool bytes = false, bits = false;
-    for (const OpDesc &d : descs) (d.bits ? bits : bytes) = true;
+    int64_t work = 0, deep = 0;   // (member, word) pairs of the bit ops, and of those in several slabs
+    for (const OpDesc &d : descs) {
+        (d.bits ? bits : bytes) = true;
+        const int64_t pairs = (int64_t)d.n * d.words_per_row * d.height;
+        work += pairs;
+        if (d.n > d.slab) deep += pairs;
+    }
     const OpDesc *ops = static_cast<const OpDesc *>(d_ops);
     const int n_ops = (int)descs.size();
     if (!bits)
         launch_accumulate_t<kBytesOnly>(e, ops, n_ops, n_items, counter);
+    else if (!bytes && e->cfg.ctas_per_sm >= kDeepBitsCtas && 2 * deep > work)
+        launch_accumulate_t<kBitsOnly, kDeepBitsCtas>(e, ops, n_ops, n_items, counter);
     else if (!bytes)
         launch_accumulate_t<kBitsOnly>(e, ops, n_ops, n_items, counter);
     else
