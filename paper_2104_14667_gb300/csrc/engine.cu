@@ -1855,11 +1855,14 @@ int composite_engine_tune(composite_engine *e, const composite_op *ops, int32_t 
     };
     // pass 1: slab depth x schedule (ctas_per_sm 0 stands for the grid schedule)
     static const int slabs[] = {32, 64, 128, 255};
-    static const int ctas[] = {0, 3, 4};
+    static const int ctas[] = {0, 3, 4, kDeepBitsCtas};
+    bool any_bits = false;
+    for (const OpDesc &d : descs) any_bits = any_bits || d.bits;
     const int ctas_before = e->cfg.ctas_per_sm;
     for (int sl : slabs)
         for (int c : ctas) {
             if (rc) break;
+            if (c == kDeepBitsCtas && !any_bits) continue;   // would run as four
             e->cfg.slab_members = sl;
             e->cfg.schedule = c ? CPT_SCHEDULE_PERSISTENT : CPT_SCHEDULE_GRID;
             e->cfg.ctas_per_sm = c ? c : ctas_before;
