@@ -46,6 +46,12 @@ def test_long_rows_of_depths(path):
         np.testing.assert_array_equal(comp.render_host()["mean"], d.sum(axis=0) / np.float32(n))
 
 
+def odd_and_even(n, h, w, pad):
+    """Depths of one pinned buffer with rows off 16-byte boundaries, and with rows (w + pad floats) on them."""
+    even = pinned(n, h, w, pad, 0, torch.float32)
+    return even.as_strided((n, h, w), ((w + 1) * h + 5, w + 1, 1)), even
+
+
 def pass_seconds(w, h, src, path) -> float:
     mean = torch.empty((h, w), dtype=torch.float32, device="cuda")
     with binding.Composite(w, h, read_path=path, mode="mean_depth") as comp:
@@ -64,8 +70,7 @@ def pass_seconds(w, h, src, path) -> float:
 
 def test_a_fold_runs_beside_the_next_upload():
     n, h, w = 16, 2048, 4090
-    odd = pinned(n, h, w, 1, 5, torch.float32)       # moved by a kernel
-    even = pinned(n, h, w, 2, 0, torch.float32)      # rows on 16-byte boundaries: pitched copies
+    odd, even = odd_and_even(n, h, w, 2)
     # several contexts: whether the folds find room had differed from one to the next
     took = [pass_seconds(w, h, odd, "tma") for _ in range(4)]
     copies = pass_seconds(w, h, even, "tma")
@@ -76,8 +81,7 @@ def test_a_fold_runs_beside_the_next_upload():
 
 def test_long_rows_take_no_longer_than_aligned_ones():
     n, h, w = 16, 1500, 6001
-    odd = pinned(n, h, w, 1, 5, torch.float32)
-    even = pinned(n, h, w, 3, 0, torch.float32)      # rows on 16-byte boundaries: pitched copies
+    odd, even = odd_and_even(n, h, w, 3)
     took = [pass_seconds(w, h, src, "linear") for src in (odd, even)]
     # 2.86 ms both; 3.35 the first when a kernel moved rows of any length
     assert took[0] < 1.07 * took[1], took
